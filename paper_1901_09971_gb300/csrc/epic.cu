@@ -25,8 +25,9 @@
 //      (every frontier seed within its smallest incoming link of the frontier
 //      minimum is final, so about 14 steps settle the 128 nearest instead of 128
 //      pops), a hash of discovered seeds in shared memory, then sorts the settled
-//      (distance, index) keys and fits the weighted affine model to the first k
-//      (double-float sums, FP64 solve). A search that outgrows the hash (384 seeds;
+//      (distance, index) keys and sums the weighted affine fit's terms over the first k
+//      (double-float); a thread per seed solves the fits (FP64). A search that outgrows
+//      the hash (384 seeds;
 //      1024 for k > 160) or the sort buffer (256; 512) is queued and redone by a
 //      retry kernel with room for 8192;
 //   10. dense flow: every pixel evaluates its seed's model.
@@ -402,29 +403,20 @@ __global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, i
     }
 }
 
-// Link records for the search: (neighbour, its list begin, its list end, its
-// smallest link weight).
-__global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(const int* off, const int* end, const int* adj_t,
-                                                                  const unsigned* minin, int4* adj_i, int n)
-{
-    const int s = blockIdx.x * kThreads + threadIdx.x;
-    if (s >= n) return;
-    for (int i = off[s], e = end[s]; i < e; ++i) {
-        const int t = adj_t[i];
-        adj_i[i] = make_int4(t, off[t], end[t], (int)minin[t]);
-    }
-}
-
 struct KnnArgs {
     const float2* pts;
     const float2* flow;
     const int* seed_pix;
     const int* off;
-    const int* end;
+    const int* end_of;
     const unsigned* minin;
     const int4* adj_i;
     const long long* adj_w;
     double* models;  // [n][6]
+    const int* list;        // the seeds that hold a pixel, in any order
+    const int* list_count;  // their number
+    double* sums;           // [end - begin][12]: the fits' weighted sums, solved by epic_solve_kernel
+    int begin, end;         // this launch's part of the list
     int* err;
     int* retry_count;
     int* retry_list;
@@ -436,6 +428,35 @@ struct KnnArgs {
     int n, k, model;
     double a_per_unit, min_spread2;  // kernel decay per unit of distance: a / (2 cost_base)
 };
+
+// Link records for the search: (neighbour, its list begin, its list end, its
+// smallest link weight); the list of the seeds that hold a pixel (in any order; a
+// warp takes its places with one atomic), and the outputs of those that do not.
+__global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, const int* adj_t, int4* adj_i, int* list,
+                                                                  int* list_count)
+{
+    const int s = blockIdx.x * kThreads + threadIdx.x, lane = threadIdx.x & 31;
+    const bool holds = s < a.n && a.seed_pix[s] >= 0;
+    const unsigned hold = __ballot_sync(0xffffffffu, holds);
+    int at = 0;
+    if (lane == 0 && hold) at = atomicAdd(list_count, __popc(hold));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (s >= a.n) return;
+    if (!holds) {
+        if (a.knn_count) a.knn_count[s] = 0;
+        if (a.fit_kind) a.fit_kind[s] = 0;
+        for (int i = 0; i < 6; ++i) {
+            a.models[6 * (size_t)s + i] = 0.0;
+            if (a.dbg_models) a.dbg_models[6 * (size_t)s + i] = 0.0;
+        }
+        return;
+    }
+    list[at + __popc(hold & ((1u << lane) - 1))] = s;
+    for (int i = a.off[s], e = a.end_of[s]; i < e; ++i) {
+        const int t = adj_t[i];
+        adj_i[i] = make_int4(t, a.off[t], a.end_of[t], (int)a.minin[t]);
+    }
+}
 
 // Per-warp shared layout of one search: a hash of HCAP discovered seeds (index,
 // tentative distance, smallest incoming link weight, settled flag), the frontier
@@ -547,15 +568,15 @@ __device__ __forceinline__ dfl to_dfl(double v)
     return {hi, __double2float_rn(v - (double)hi)};
 }
 
-// Sums of 12 values over the warp; the totals land in lane 0. Halving exchanges:
-// lanes 16 apart swap half of their values and keep the sum of the other half, then
-// lanes 8 apart the same with 3 of 6, then xor butterflies finish the 3 sums in each
-// group of 8 lanes; lanes 8, 16 and 24 hand their 3 totals to lane 0.
-__device__ __forceinline__ void warp_sum12(const double (&v)[12], double (&out)[12])
+// Sums of 12 values over the warp: lane 8 g holds totals 3 g .. 3 g + 2 in q (other
+// lanes partial sums). Halving exchanges: lanes 16 apart swap half of their values and
+// keep the sum of the other half, then lanes 8 apart the same with 3 of 6, then xor
+// butterflies finish the 3 sums in each group of 8 lanes.
+__device__ __forceinline__ void warp_sum12(const double (&v)[12], double (&q)[3])
 {
     const int lane = threadIdx.x & 31;
     const bool hi16 = lane & 16, hi8 = lane & 8;
-    double h[6], q[3];
+    double h[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
         const double keep = hi16 ? v[6 + i] : v[i], give = hi16 ? v[i] : v[6 + i];
@@ -570,13 +591,6 @@ __device__ __forceinline__ void warp_sum12(const double (&v)[12], double (&out)[
     for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
         for (int i = 0; i < 3; ++i) q[i] += __shfl_xor_sync(0xffffffffu, q[i], o);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        out[i] = q[i];
-        out[3 + i] = __shfl_sync(0xffffffffu, q[i], 8);
-        out[6 + i] = __shfl_sync(0xffffffffu, q[i], 16);
-        out[9 + i] = __shfl_sync(0xffffffffu, q[i], 24);
-    }
 }
 
 __device__ __forceinline__ long long warp_min64(long long v)  // v >= 0
@@ -707,7 +721,7 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
                 u = (int)(kb & kIdxMask);
                 du = (long long)(kb >> kIdxBits);
                 first = a.off[u];
-                deg = a.end[u] - first;
+                deg = a.end_of[u] - first;
             }
             int incl = deg;
 #pragma unroll
@@ -790,12 +804,13 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
     return status & kErrRange ? kErrRange : status;
 }
 
-// The weighted affine fit of seed s over its neighbourhood (sorted keys) and the
-// outputs. The 3 x 3 normal equations lose too many digits in FP32 when a
-// neighbourhood is narrow: the weights come from an FP64 exponential, the
+// The weighted sums of the affine fit of seed s (entry idx of the list) over its neighbourhood (sorted keys), and
+// the neighbourhood outputs. The 3 x 3 normal equations lose too many digits in FP32
+// when a neighbourhood is narrow: the weights come from an FP64 exponential, the
 // per-neighbour terms are summed in double-float, the lanes' sums are reduced and
-// the systems solved in FP64. M = sum w v v^T, v = (x_t - x_s, y_t - y_s, 1).
-__device__ void knn_fit_write(const KnnArgs& a, int s, int cnt, const unsigned long long* key)
+// the systems solved in FP64 (epic_solve_kernel). M = sum w v v^T,
+// v = (x_t - x_s, y_t - y_s, 1).
+__device__ void knn_fit_sums(const KnnArgs& a, int idx, int s, int cnt, const unsigned long long* key)
 {
     const int lane = threadIdx.x & 31, k = a.k;
     if (a.knn_count && lane == 0) a.knn_count[s] = cnt;
@@ -830,14 +845,32 @@ __device__ void knn_fit_write(const KnnArgs& a, int s, int cnt, const unsigned l
     double accd[12];
 #pragma unroll
     for (int i = 0; i < 12; ++i) accd[i] = (double)acc[i].hi + (double)acc[i].lo;
-    double tot[12];
+    double tot[3];
     warp_sum12(accd, tot);
-    if (lane != 0) return;
-    const double m00 = tot[0], m01 = tot[1], m02 = tot[2], m11 = tot[3], m12 = tot[4], m22 = tot[5];
-    const double u0 = tot[6], u1 = tot[7], u2 = tot[8], v0 = tot[9], v1 = tot[10], v2 = tot[11];
+    if (lane & 7) return;
+    double* row = a.sums + 12 * (size_t)(idx - a.begin) + 3 * (lane >> 3);
+    row[0] = tot[0];
+    row[1] = tot[1];
+    row[2] = lane == 8 && cnt < 3 ? -tot[2] : tot[2];  // sum w > 0: a negative one marks fewer than 3 neighbours
+}
+
+// Solves the fits of this launch's seeds from their sums, a thread a seed. The
+// solve is about 250 FP64 operations (a dozen divisions and square roots); GB300
+// issues an FP64 instruction of one lane no faster than one of 32, so on lane 0 of
+// each search's warp the solves kept the search kernel's FP64 pipe busy 58% of its
+// time. 1242x375 pair, 50,676 matches, k = 128: a call 1,761 -> 1,301 us.
+__global__ void __launch_bounds__(kThreads) epic_solve_kernel(KnnArgs a)
+{
+    const int idx = a.begin + blockIdx.x * kThreads + threadIdx.x;
+    if (idx >= min(a.end, *a.list_count)) return;
+    const int s = a.list[idx];
+    const double2* row = reinterpret_cast<const double2*>(a.sums + 12 * (size_t)(idx - a.begin));
+    const double2 q0 = row[0], q1 = row[1], q2 = row[2], q3 = row[3], q4 = row[4], q5 = row[5];
+    const double m00 = q0.x, m01 = q0.y, m02 = q1.x, m11 = q1.y, m12 = q2.x, m22 = fabs(q2.y);
+    const double u0 = q3.x, u1 = q3.y, u2 = q4.x, v0 = q4.y, v1 = q5.x, v2 = q5.y;
     // affine only with 3+ neighbours whose weighted position covariance (the Schur
     // complement of the constant term over sum w) has lambda_min >= min_spread^2
-    bool affine = a.model == 1 && cnt >= 3;
+    bool affine = a.model == 1 && q2.y > 0.0;
     if (affine) {
         const double mx = m02 / m22, my = m12 / m22;
         const double cxx = m00 / m22 - mx * mx, cxy = m01 / m22 - mx * my, cyy = m11 / m22 - my * my;
@@ -876,48 +909,41 @@ __global__ void __launch_bounds__(kFastWarps * 32) epic_knn_fit_kernel(KnnArgs a
     using Lay = KnnLayout<HCAP, FCAP, SCAP>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int s = blockIdx.x * kFastWarps + wid;
-    if (s >= a.n) return;  // warp-uniform
-    if (a.seed_pix[s] < 0) {
-        if (lane == 0) {
-            if (a.knn_count) a.knn_count[s] = 0;
-            if (a.fit_kind) a.fit_kind[s] = 0;
-        }
-        if (lane < 6) {
-            a.models[6 * (size_t)s + lane] = 0.0;
-            if (a.dbg_models) a.dbg_models[6 * (size_t)s + lane] = 0.0;
-        }
-        return;
-    }
+    const int idx = a.begin + blockIdx.x * kFastWarps + wid;
+    if (idx >= min(a.end, *a.list_count)) return;  // warp-uniform
+    const int s = a.list[idx];
     unsigned char* base = smem + (size_t)wid * Lay::bytes;
     int cnt = 0;
     const int st = knn_search<HCAP, FCAP, SCAP>(a, s, base, cnt);
     if (st == kRetry) {
-        if (lane == 0) a.retry_list[atomicAdd(a.retry_count, 1)] = s;
+        if (lane == 0) a.retry_list[atomicAdd(a.retry_count, 1)] = idx;
         return;
     }
     if (st) {
         if (lane == 0) atomicOr(a.err, st);
         return;
     }
-    knn_fit_write(a, s, cnt, reinterpret_cast<const unsigned long long*>(base + Lay::o_sort));
+    knn_fit_sums(a, idx, s, cnt, reinterpret_cast<const unsigned long long*>(base + Lay::o_sort));
 }
 
-// The queued searches with room for 8192 discovered seeds, one warp per block.
+// The queued searches of this launch's seeds with room for 8192 discovered seeds, one
+// warp per block.
 __global__ void __launch_bounds__(32) epic_knn_retry_kernel(KnnArgs a)
 {
     using Lay = KnnLayout<kBigH, kBigF, kBigS>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int total = *a.retry_count;
     for (int i = blockIdx.x; i < total; i += gridDim.x) {
-        const int s = a.retry_list[i];
+        const int idx = a.retry_list[i];
+        if (idx < a.begin) continue;  // of an earlier launch
+        const int s = a.list[idx];
         int cnt = 0;
         const int st = knn_search<kBigH, kBigF, kBigS>(a, s, smem, cnt);
         if (st) {
             if ((threadIdx.x & 31) == 0) atomicOr(a.err, st == kRetry ? kErrFrontier : st);
             continue;
         }
-        knn_fit_write(a, s, cnt, reinterpret_cast<const unsigned long long*>(smem + Lay::o_sort));
+        knn_fit_sums(a, idx, s, cnt, reinterpret_cast<const unsigned long long*>(smem + Lay::o_sort));
     }
 }
 
@@ -943,6 +969,9 @@ __global__ void __launch_bounds__(kThreads) epic_dense_kernel(const unsigned lon
     if (labels) labels[o] = s;
     if (dist) dist[o] = (int64_t)(k >> kIdxBits);
 }
+
+// Pass counters, the status word, the retry count, the barrier, the list's length.
+constexpr int kCounters = kMaxPasses + 4;
 
 // Workspace layout (256-byte aligned sections).
 struct EpicLayout {
@@ -972,7 +1001,7 @@ EpicLayout epic_layout(int W, int H, int n)
     L.adj_i = take(nl * 16);
     L.models = take((size_t)n * 48);
     L.retry = take((size_t)n * 4);
-    L.counters = take((kMaxPasses + 3) * 4);  // pass counters, the status word, the retry count, the barrier
+    L.counters = take(kCounters * 4);
     L.total = at;
     return L;
 }
@@ -1061,12 +1090,13 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
     int* err = changed + kMaxPasses;
     int* retry_count = err + 1;
     unsigned* sync_count = reinterpret_cast<unsigned*>(retry_count + 1);
+    int* list_count = retry_count + 2;
     const float2* p2 = reinterpret_cast<const float2*>(pts);
     const float2* f2 = reinterpret_cast<const float2*>(flow);
 
     unsigned* dev_status = dgf::status_word();
     if (!dev_status) return DGF_ERR_CUDA;
-    if (cudaMemsetAsync(changed, 0, (kMaxPasses + 3) * sizeof(int), stream) != cudaSuccess) return DGF_ERR_CUDA;
+    if (cudaMemsetAsync(changed, 0, kCounters * sizeof(int), stream) != cudaSuccess) return DGF_ERR_CUDA;
     if (n > 0 && cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(int), stream) != cudaSuccess) return DGF_ERR_CUDA;
     const dim3 pix_block(32, 8), pix_grid((W + 31) / 32, (H + 7) / 8);
     const unsigned pt_grid = (unsigned)((n + kThreads - 1) / kThreads);
@@ -1108,13 +1138,12 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
                                                                     err);
         epic_dedupe_kernel<<<(unsigned)((n + kThreads / 32 - 1) / (kThreads / 32)), kThreads, 0, stream>>>(
             off, cur, adj_t, adj_w, minin, n);
-        epic_link_meta_kernel<<<pt_grid, kThreads, 0, stream>>>(off, cur, adj_t, minin, adj_i, n);
         KnnArgs a;
         a.pts = p2;
         a.flow = f2;
         a.seed_pix = seed_pix;
         a.off = off;
-        a.end = cur;
+        a.end_of = cur;
         a.minin = minin;
         a.adj_i = adj_i;
         a.adj_w = adj_w;
@@ -1145,8 +1174,24 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
             return DGF_ERR_CUDA;
-        fast<<<(unsigned)((n + kFastWarps - 1) / kFastWarps), kFastWarps * 32, smem_fast, stream>>>(a);
-        epic_knn_retry_kernel<<<(unsigned)sms, 32, smem_big, stream>>>(a);
+        // the list takes the place of the link counts; the fits' sums that of adj_t once
+        // the link records are made. Seeds beyond its room (W H / 6 of them; at most
+        // W H hold a pixel) are searched and solved in further launches.
+        int* list = cnt;
+        a.list = list;
+        a.list_count = list_count;
+        epic_link_meta_kernel<<<pt_grid, kThreads, 0, stream>>>(a, adj_t, adj_i, list, list_count);
+        a.sums = reinterpret_cast<double*>(adj_t);
+        const long long holders = std::min<long long>(n, (long long)W * H);
+        const long long room = (long long)((L.adj_w - L.adj_t) / (12 * sizeof(double)));
+        for (long long at = 0; at < holders; at += room) {
+            a.begin = (int)at;
+            a.end = (int)std::min(holders, at + room);
+            const int m = a.end - a.begin;
+            fast<<<(unsigned)((m + kFastWarps - 1) / kFastWarps), kFastWarps * 32, smem_fast, stream>>>(a);
+            epic_knn_retry_kernel<<<(unsigned)sms, 32, smem_big, stream>>>(a);
+            epic_solve_kernel<<<(unsigned)((m + kThreads - 1) / kThreads), kThreads, 0, stream>>>(a);
+        }
     }
     epic_dense_kernel<<<pix_grid, pix_block, 0, stream>>>(key, models, p2, W, H, reinterpret_cast<float2*>(dense),
                                                           d.labels, d.dist);
