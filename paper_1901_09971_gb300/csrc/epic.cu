@@ -347,62 +347,6 @@ __global__ void __launch_bounds__(1024) epic_scan_add_kernel(const int* boff, in
     if (i == 0) off[n] = boff[nb];
 }
 
-// Per seed: keeps one link per neighbour (the smallest weight), compacting the list
-// in place; end[s] becomes the end of the compacted list. One warp per seed walks
-// the list in chunks of 32: lanes holding the same neighbour find each other with
-// match.any and take their minimum weight; the lowest of them either lowers the
-// weight of a link kept from an earlier chunk or appends a new one. The kept prefix
-// never reaches the unread part of the list.
-__global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, int* end, int* adj_t, long long* adj_w,
-                                                               unsigned* minin, int n)
-{
-    const int lane = threadIdx.x & 31;
-    const int s = (int)(((size_t)blockIdx.x * kThreads + threadIdx.x) >> 5);
-    if (s >= n) return;  // warp-uniform
-    const int b = off[s], e = off[s + 1];
-    int out = b;
-    for (int c = b; c < e; c += 32) {
-        const bool has = c + lane < e;
-        const int t = has ? adj_t[c + lane] : -1 - lane;  // empty lanes match nobody
-        const long long w = has ? adj_w[c + lane] : 0;
-        const unsigned grp = __match_any_sync(0xffffffffu, t);
-        long long mw = w;
-        for (int j = 0; j < 32; ++j) {
-            const long long wj = __shfl_sync(0xffffffffu, w, j);
-            if ((grp >> j) & 1u) mw = min(mw, wj);
-        }
-        const bool leader = has && lane == __ffs(grp) - 1;
-        int found = -1;
-        if (leader)
-            for (int j = b; j < out; ++j)
-                if (adj_t[j] == t) {
-                    found = j;
-                    break;
-                }
-        if (found >= 0 && mw < adj_w[found]) adj_w[found] = mw;  // leaders hold distinct neighbours
-        const bool app = leader && found < 0;
-        const unsigned km = __ballot_sync(0xffffffffu, app);
-        __syncwarp();
-        if (app) {
-            const int pos = out + __popc(km & ((1u << lane) - 1));
-            adj_t[pos] = t;
-            adj_w[pos] = mw;
-        }
-        out += __popc(km);
-        __syncwarp();
-    }
-    // smallest link weight (a lower bound on the last step of any path into s),
-    // clamped to 32 bits (a smaller bound stays a bound)
-    long long mn = kNoLink;
-    for (int j = b + lane; j < out; j += 32) mn = min(mn, adj_w[j]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    if (lane == 0) {
-        end[s] = out;
-        minin[s] = (unsigned)min(mn, (long long)kNoLink);
-    }
-}
-
 struct KnnArgs {
     const float2* pts;
     const float2* flow;
@@ -417,6 +361,8 @@ struct KnnArgs {
     const int* list_count;  // their number
     double* sums;           // [end - begin][12]: the fits' weighted sums, solved by epic_solve_kernel
     int begin, end;         // this launch's part of the list
+    const float2* weights;  // [n_weights]: the fit weights of distances 0 .. n_weights - 1 (double-float)
+    int n_weights;
     int* err;
     int* retry_count;
     int* retry_list;
@@ -428,35 +374,6 @@ struct KnnArgs {
     int n, k, model;
     double a_per_unit, min_spread2;  // kernel decay per unit of distance: a / (2 cost_base)
 };
-
-// Link records for the search: (neighbour, its list begin, its list end, its
-// smallest link weight); the list of the seeds that hold a pixel (in any order; a
-// warp takes its places with one atomic), and the outputs of those that do not.
-__global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, const int* adj_t, int4* adj_i, int* list,
-                                                                  int* list_count)
-{
-    const int s = blockIdx.x * kThreads + threadIdx.x, lane = threadIdx.x & 31;
-    const bool holds = s < a.n && a.seed_pix[s] >= 0;
-    const unsigned hold = __ballot_sync(0xffffffffu, holds);
-    int at = 0;
-    if (lane == 0 && hold) at = atomicAdd(list_count, __popc(hold));
-    at = __shfl_sync(0xffffffffu, at, 0);
-    if (s >= a.n) return;
-    if (!holds) {
-        if (a.knn_count) a.knn_count[s] = 0;
-        if (a.fit_kind) a.fit_kind[s] = 0;
-        for (int i = 0; i < 6; ++i) {
-            a.models[6 * (size_t)s + i] = 0.0;
-            if (a.dbg_models) a.dbg_models[6 * (size_t)s + i] = 0.0;
-        }
-        return;
-    }
-    list[at + __popc(hold & ((1u << lane) - 1))] = s;
-    for (int i = a.off[s], e = a.end_of[s]; i < e; ++i) {
-        const int t = adj_t[i];
-        adj_i[i] = make_int4(t, a.off[t], a.end_of[t], (int)a.minin[t]);
-    }
-}
 
 // Per-warp shared layout of one search: a hash of HCAP discovered seeds (index,
 // tentative distance, smallest incoming link weight, settled flag), the frontier
@@ -568,6 +485,18 @@ __device__ __forceinline__ dfl to_dfl(double v)
     return {hi, __double2float_rn(v - (double)hi)};
 }
 
+// The fit weight of a neighbour at distance d. Distances are integers, so the weights
+// of the first kWeights come from a table that each call fills once: at k = 128 the
+// search evaluated 128 FP64 exponentials a seed (about 20 instructions of the narrow
+// FP64 pipe each) for a few thousand distinct distances. The table's entries are this
+// function's values; weights past its end (exp(-205) at the default decay) are
+// computed. A call on the 1242x375 pair 1,301 -> 1,231 us.
+constexpr int kWeights = 16384;
+__device__ __forceinline__ dfl fit_weight(double a_per_unit, long long d)
+{
+    return to_dfl(exp_neg(a_per_unit * (double)d));
+}
+
 // Sums of 12 values over the warp: lane 8 g holds totals 3 g .. 3 g + 2 in q (other
 // lanes partial sums). Halving exchanges: lanes 16 apart swap half of their values and
 // keep the sum of the other half, then lanes 8 apart the same with 3 of 6, then xor
@@ -591,6 +520,97 @@ __device__ __forceinline__ void warp_sum12(const double (&v)[12], double (&q)[3]
     for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
         for (int i = 0; i < 3; ++i) q[i] += __shfl_xor_sync(0xffffffffu, q[i], o);
+}
+
+// Per seed: keeps one link per neighbour (the smallest weight), compacting the list
+// in place; end[s] becomes the end of the compacted list. One warp per seed walks
+// the list in chunks of 32: lanes holding the same neighbour find each other with
+// match.any and take their minimum weight; the lowest of them either lowers the
+// weight of a link kept from an earlier chunk or appends a new one. The kept prefix
+// never reaches the unread part of the list. Also fills the table of fit weights, an
+// entry a thread.
+__global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, int* end, int* adj_t, long long* adj_w,
+                                                               unsigned* minin, int n, double a_per_unit, float2* weights,
+                                                               int n_weights)
+{
+    for (int d = blockIdx.x * kThreads + threadIdx.x; d < n_weights; d += gridDim.x * kThreads) {
+        const dfl w = fit_weight(a_per_unit, d);
+        weights[d] = make_float2(w.hi, w.lo);
+    }
+    const int lane = threadIdx.x & 31;
+    const int s = (int)(((size_t)blockIdx.x * kThreads + threadIdx.x) >> 5);
+    if (s >= n) return;  // warp-uniform
+    const int b = off[s], e = off[s + 1];
+    int out = b;
+    for (int c = b; c < e; c += 32) {
+        const bool has = c + lane < e;
+        const int t = has ? adj_t[c + lane] : -1 - lane;  // empty lanes match nobody
+        const long long w = has ? adj_w[c + lane] : 0;
+        const unsigned grp = __match_any_sync(0xffffffffu, t);
+        long long mw = w;
+        for (int j = 0; j < 32; ++j) {
+            const long long wj = __shfl_sync(0xffffffffu, w, j);
+            if ((grp >> j) & 1u) mw = min(mw, wj);
+        }
+        const bool leader = has && lane == __ffs(grp) - 1;
+        int found = -1;
+        if (leader)
+            for (int j = b; j < out; ++j)
+                if (adj_t[j] == t) {
+                    found = j;
+                    break;
+                }
+        if (found >= 0 && mw < adj_w[found]) adj_w[found] = mw;  // leaders hold distinct neighbours
+        const bool app = leader && found < 0;
+        const unsigned km = __ballot_sync(0xffffffffu, app);
+        __syncwarp();
+        if (app) {
+            const int pos = out + __popc(km & ((1u << lane) - 1));
+            adj_t[pos] = t;
+            adj_w[pos] = mw;
+        }
+        out += __popc(km);
+        __syncwarp();
+    }
+    // smallest link weight (a lower bound on the last step of any path into s),
+    // clamped to 32 bits (a smaller bound stays a bound)
+    long long mn = kNoLink;
+    for (int j = b + lane; j < out; j += 32) mn = min(mn, adj_w[j]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    if (lane == 0) {
+        end[s] = out;
+        minin[s] = (unsigned)min(mn, (long long)kNoLink);
+    }
+}
+
+// Link records for the search: (neighbour, its list begin, its list end, its
+// smallest link weight); the list of the seeds that hold a pixel (in any order; a
+// warp takes its places with one atomic), and the outputs of those that do not.
+__global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, const int* adj_t, int4* adj_i, int* list,
+                                                                  int* list_count)
+{
+    const int s = blockIdx.x * kThreads + threadIdx.x, lane = threadIdx.x & 31;
+    const bool holds = s < a.n && a.seed_pix[s] >= 0;
+    const unsigned hold = __ballot_sync(0xffffffffu, holds);
+    int at = 0;
+    if (lane == 0 && hold) at = atomicAdd(list_count, __popc(hold));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (s >= a.n) return;
+    if (!holds) {
+        if (a.knn_count) a.knn_count[s] = 0;
+        if (a.fit_kind) a.fit_kind[s] = 0;
+        for (int i = 0; i < 6; ++i) {
+            a.models[6 * (size_t)s + i] = 0.0;
+            if (a.dbg_models) a.dbg_models[6 * (size_t)s + i] = 0.0;
+        }
+        return;
+    }
+    list[at + __popc(hold & ((1u << lane) - 1))] = s;
+    for (int i = a.off[s], e = a.end_of[s]; i < e; ++i) {
+        const int t = adj_t[i];
+        adj_i[i] = make_int4(t, a.off[t], a.end_of[t], (int)a.minin[t]);
+    }
 }
 
 __device__ __forceinline__ long long warp_min64(long long v)  // v >= 0
@@ -825,7 +845,14 @@ __device__ void knn_fit_sums(const KnnArgs& a, int idx, int s, int cnt, const un
     for (int i = 0; i < 12; ++i) acc[i] = {0.f, 0.f};
     for (int j = lane; j < cnt; j += 32) {
         const int t = (int)(key[j] & kIdxMask);
-        const dfl w = to_dfl(exp_neg(a.a_per_unit * (double)(long long)(key[j] >> kIdxBits)));
+        const long long d = (long long)(key[j] >> kIdxBits);
+        dfl w;
+        if (d < a.n_weights) {
+            const float2 t = __ldg(a.weights + d);
+            w = {t.x, t.y};
+        } else {
+            w = fit_weight(a.a_per_unit, d);
+        }
         const float2 pt = a.pts[t], ft = a.flow[t];
         const dfl vx = two_sum(pt.x, -ps.x), vy = two_sum(pt.y, -ps.y);  // exact differences
         const dfl wx = df_mul(w, vx), wy = df_mul(w, vy);
@@ -1136,8 +1163,10 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         epic_scan_add_kernel<<<nb, 1024, 0, stream>>>(bsum + nb, n, nb, off, cur);
         epic_links_kernel<true><<<pix_grid, pix_block, 0, stream>>>(key, cost, W, H, nullptr, off, cur, adj_t, adj_w,
                                                                     err);
+        // the weights' table takes the place of the pixel costs
+        const int n_weights = (int)std::min<size_t>(kWeights, (L.seed_pix - L.cost) / sizeof(float2));
         epic_dedupe_kernel<<<(unsigned)((n + kThreads / 32 - 1) / (kThreads / 32)), kThreads, 0, stream>>>(
-            off, cur, adj_t, adj_w, minin, n);
+            off, cur, adj_t, adj_w, minin, n, p->a / (2.0 * p->cost_base), reinterpret_cast<float2*>(cost), n_weights);
         KnnArgs a;
         a.pts = p2;
         a.flow = f2;
@@ -1180,6 +1209,8 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         int* list = cnt;
         a.list = list;
         a.list_count = list_count;
+        a.n_weights = n_weights;
+        a.weights = reinterpret_cast<const float2*>(cost);
         epic_link_meta_kernel<<<pt_grid, kThreads, 0, stream>>>(a, adj_t, adj_i, list, list_count);
         a.sums = reinterpret_cast<double*>(adj_t);
         const long long holders = std::min<long long>(n, (long long)W * H);
