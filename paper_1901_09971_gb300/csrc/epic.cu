@@ -354,8 +354,7 @@ struct KnnArgs {
     const int* off;
     const int* end_of;
     const unsigned* minin;
-    const int4* adj_i;
-    const long long* adj_w;
+    const int4* adj;  // link records: neighbour, its smallest link weight, the link's weight (low, high)
     double* models;  // [n][6]
     const int* list;        // the seeds that hold a pixel, in any order
     const int* list_count;  // their number
@@ -376,17 +375,19 @@ struct KnnArgs {
 };
 
 // Per-warp shared layout of one search: a hash of HCAP discovered seeds (index,
-// tentative distance, smallest incoming link weight, settled flag), the frontier
-// as a list of FCAP hash slots, and the settled keys (SCAP, later sorted in place).
-template <int HCAP, int FCAP, int SCAP>
+// tentative distance, smallest incoming link weight), the frontier as a list of FCAP
+// hash slots, and the settled keys (SCAP, later sorted in place). Distances are of
+// type DT: 32 bits in the fast layouts (half the shared traffic of 64, and a native
+// shared atomic minimum where a 64-bit one is a compare-and-swap loop), 64 in the
+// retry kernel's.
+template <typename DT, int HCAP, int FCAP, int SCAP>
 struct KnnLayout {
-    static_assert(HCAP % 32 == 0 && (SCAP & (SCAP - 1)) == 0 && HCAP <= 32768, "sizes");
+    static_assert(HCAP % 128 == 0 && SCAP % 32 == 0 && HCAP <= 32768, "sizes");
     static constexpr size_t o_hdist = (size_t)HCAP * 4;
-    static constexpr size_t o_sort = o_hdist + (size_t)HCAP * 8;
+    static constexpr size_t o_sort = o_hdist + (size_t)HCAP * sizeof(DT);
     static constexpr size_t o_minin = o_sort + (size_t)SCAP * 8;
     static constexpr size_t o_front = o_minin + (size_t)HCAP * 4;
-    static constexpr size_t o_state = o_front + (size_t)FCAP * 2;
-    static constexpr size_t o_count = (o_state + (size_t)HCAP + 15) & ~(size_t)15;
+    static constexpr size_t o_count = (o_front + (size_t)FCAP * 2 + 15) & ~(size_t)15;
     static constexpr size_t bytes = o_count + 16;
 };
 
@@ -395,10 +396,11 @@ struct KnnLayout {
 // the larger one); a search that outgrows them is redone by the retry kernel with
 // room for 8192.
 constexpr int kFastWarps = 4, kSmallK = 160;
+using SmallLayout = KnnLayout<unsigned, 384, 256, 256>;
+using LargeLayout = KnnLayout<unsigned, 1024, 512, 512>;
 constexpr int kBigH = 8192, kBigF = 8192, kBigS = 8192;  // the retry kernel runs one block per SM
+using RetryLayout = KnnLayout<long long, kBigH, kBigF, kBigS>;
 constexpr int kRetry = 16;  // search status: capacity exceeded, redo with the large layout
-constexpr long long kInf = 0x7fffffffffffffffll;
-enum : unsigned char { kFrontier = 0, kSettled = 1 };
 
 // exp(-y) for y >= 0 by the table-driven method of Tang (ACM TOMS 15(2), 1989):
 // y = (32 q + j) ln2 / 32 + r with |r| <= ln2 / 64, so exp(-y) = 2^-q 2^(-j/32)
@@ -584,10 +586,11 @@ __global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, i
     }
 }
 
-// Link records for the search: (neighbour, its list begin, its list end, its
-// smallest link weight); the list of the seeds that hold a pixel (in any order; a
+// Link records for the search (one 16-byte load a link): neighbour, its smallest link
+// weight, the link's weight; the list of the seeds that hold a pixel (in any order; a
 // warp takes its places with one atomic), and the outputs of those that do not.
-__global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, const int* adj_t, int4* adj_i, int* list,
+__global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, const int* adj_t,
+                                                                  const long long* adj_w, int4* adj, int* list,
                                                                   int* list_count)
 {
     const int s = blockIdx.x * kThreads + threadIdx.x, lane = threadIdx.x & 31;
@@ -609,34 +612,111 @@ __global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, con
     list[at + __popc(hold & ((1u << lane) - 1))] = s;
     for (int i = a.off[s], e = a.end_of[s]; i < e; ++i) {
         const int t = adj_t[i];
-        adj_i[i] = make_int4(t, a.off[t], a.end_of[t], (int)a.minin[t]);
+        const long long w = adj_w[i];
+        adj[i] = make_int4(t, (int)a.minin[t], (int)(unsigned)w, (int)(w >> 32));
     }
 }
 
-__device__ __forceinline__ long long warp_min64(long long v)  // v >= 0
+__device__ __forceinline__ long long warp_min(long long v)  // v >= 0
 {
     const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)((unsigned long long)v >> 32));
     const unsigned lo = __reduce_min_sync(0xffffffffu, (unsigned)((unsigned long long)v >> 32) == hi ? (unsigned)v : ~0u);
     return (long long)(((unsigned long long)hi << 32) | lo);
 }
+__device__ __forceinline__ unsigned warp_min(unsigned v) { return __reduce_min_sync(0xffffffffu, v); }
 
-// Ascending bitonic sort of N keys (a power of two) in shared memory by one warp.
-__device__ void warp_bitonic_sort(unsigned long long* key, int N)
+__device__ __forceinline__ void atomic_min_shared(long long* p, long long v)
+{
+    atomicMin(reinterpret_cast<unsigned long long*>(p), (unsigned long long)v);  // v >= 0
+}
+__device__ __forceinline__ void atomic_min_shared(unsigned* p, unsigned v) { atomicMin(p, v); }
+
+// Ascending sort of the first n <= 32 P keys of a shared array by one warp: P keys a
+// lane in registers (lane l holds elements P l .. P l + P - 1), a bitonic network whose
+// strides below P stay in the lane and whose others are shuffles. Slots past n are
+// filled with the largest key and not written back.
+template <int P>
+__device__ __forceinline__ void warp_sort(unsigned long long* key, int n)
 {
     const int lane = threadIdx.x & 31;
-    for (int size = 2; size <= N; size <<= 1)
+    unsigned long long v[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) v[i] = lane + 32 * i < n ? key[lane + 32 * i] : kNone;  // any order will do
+#pragma unroll
+    for (int size = 2; size <= 32 * P; size <<= 1)
+#pragma unroll
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = lane; i < N / 2; i += 32) {
-                const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
-                const bool asc = (lo & size) == 0;
-                const unsigned long long x = key[lo], y = key[hi];
-                if ((x > y) == asc) {
-                    key[lo] = y;
-                    key[hi] = x;
+            if (stride >= P) {
+                // element e's partner e ^ stride is element i of lane ^ (stride / P)
+                const int o = stride / P;
+                const bool low = (lane & o) == 0, asc = size < 32 * P ? ((lane * P) & size) == 0 : true;
+#pragma unroll
+                for (int i = 0; i < P; ++i) {
+                    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v[i], o);
+                    v[i] = (v[i] < w) == (low == asc) ? v[i] : w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < P; ++i) {
+                    if (i & stride) continue;
+                    const bool asc = size < P ? (i & size) == 0 : size < 32 * P ? ((lane * P) & size) == 0 : true;
+                    const unsigned long long x = v[i], y = v[i ^ stride];
+                    const bool keep = (x < y) == asc;
+                    v[i] = keep ? x : y;
+                    v[i ^ stride] = keep ? y : x;
                 }
             }
-            __syncwarp();
         }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+        if (P * lane + i < n) key[P * lane + i] = v[i];
+    __syncwarp();
+}
+
+// Moves the `want` smallest of n distinct keys (want < n) to the front of a shared
+// array, in any order. The want-th smallest distance is found by bisection between
+// lo and hi (fewer than want keys lie below lo, at least want at or below hi), then,
+// if more than want keys are at or below it, the index bound among those at it.
+__device__ __forceinline__ void warp_select(unsigned long long* key, int n, int want, long long lo, long long hi)
+{
+    const int lane = threadIdx.x & 31;
+    auto count = [&](unsigned long long bound) {  // keys below bound
+        int c = 0;
+        for (int i = lane; i < n; i += 32) c += key[i] < bound;
+        return (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
+    };
+    auto above = [](long long d) {  // above every key at distance d
+        return d + 1 < kDistLimit ? (unsigned long long)(d + 1) << kIdxBits : kNone;
+    };
+    while (lo < hi) {
+        const long long mid = lo + ((hi - lo) >> 1);
+        if (count(above(mid)) >= want)
+            hi = mid;
+        else
+            lo = mid + 1;
+    }
+    unsigned long long bound = above(lo);  // keys below it are kept
+    if (count(bound) > want) {
+        unsigned long long a = (unsigned long long)lo << kIdxBits, b = bound;  // count(a) < want < count(b)
+        while (a < b) {
+            const unsigned long long mid = a + ((b - a) >> 1);
+            if (count(mid) >= want)
+                b = mid;
+            else
+                a = mid + 1;
+        }
+        bound = a;
+    }
+    int kept = 0;
+    for (int c = 0; c < n; c += 32) {  // in place: kept never passes the chunk being read
+        const unsigned long long v = c + lane < n ? key[c + lane] : kNone;
+        const bool take = v < bound;
+        const unsigned tm = __ballot_sync(0xffffffffu, take);
+        if (take) key[kept + __popc(tm & ((1u << lane) - 1))] = v;
+        kept += __popc(tm);
+        __syncwarp();
+    }
 }
 
 // The k nearest seeds of seed s in the seed graph, exactly, by Dijkstra with batch
@@ -644,23 +724,31 @@ __device__ void warp_bitonic_sort(unsigned long long* key, int N)
 // seed v with d(v) <= m + minin(v) is final (a shorter path would have to end with
 // a link from an unsettled seed, at least m away, and that link weighs at least
 // minin(v)); the whole batch is settled (appended to the settled keys and removed
-// from the frontier list), then its links are relaxed, one lane per batch seed;
+// from the frontier list), then its links are relaxed, one lane per link;
 // newly discovered seeds join the frontier list. The search stops once k settled
 // seeds lie below m (every unsettled seed is at least m away) or the frontier is
-// empty; the settled keys (distance << 24 | index) are then sorted and the first
-// k kept (cnt_out). Returns 0, kRetry when the hash, the frontier list or the
-// settled list is full, or kErrRange when a distance leaves 40 bits.
-template <int HCAP, int FCAP, int SCAP>
+// empty; the k smallest settled keys (distance << 24 | index) are then selected and
+// sorted (cnt_out of them). Returns 0, kRetry when the hash, the frontier list, the
+// settled list or the distance type is too small, or kErrRange when a distance leaves
+// 40 bits.
+// Bound by instruction issue and shared-memory latency, so the steps are kept short:
+// distances of 32 bits, one 16-byte record a link, owners of links by bit masks instead
+// of a shuffled binary search, settled keys counted only once there are k of them, and
+// a register sort of the k kept keys instead of a shared-memory sort of all settled ones
+// padded to 256. Search kernel on the 1242x375 pair (k = 128): 880 -> 660 us; 28
+// searches an SM instead of 24.
+template <typename DT, int HCAP, int FCAP, int SCAP>
 __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt_out)
 {
-    using Lay = KnnLayout<HCAP, FCAP, SCAP>;
+    using Lay = KnnLayout<DT, HCAP, FCAP, SCAP>;
+    constexpr bool kNarrow = sizeof(DT) == 4;
+    constexpr DT kInf = kNarrow ? (DT)0xffffffffu : (DT)0x7fffffffffffffffll;
     int* hkey = reinterpret_cast<int*>(base);
     volatile int* vh = hkey;
-    long long* hdist = reinterpret_cast<long long*>(base + Lay::o_hdist);
+    DT* hdist = reinterpret_cast<DT*>(base + Lay::o_hdist);
     unsigned long long* skey = reinterpret_cast<unsigned long long*>(base + Lay::o_sort);
     unsigned* hmin = reinterpret_cast<unsigned*>(base + Lay::o_minin);
     short* front = reinterpret_cast<short*>(base + Lay::o_front);
-    unsigned char* hst = base + Lay::o_state;
     int* fcount = reinterpret_cast<int*>(base + Lay::o_count);  // frontier list length
     const int lane = threadIdx.x & 31;
     // multiplicative hash scaled onto [0, HCAP) (HCAP need not be a power of two)
@@ -668,10 +756,12 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
         return (int)(((unsigned long long)((unsigned)t * 0x9E3779B1u) * (unsigned)HCAP) >> 32);
     };
 
-    for (int j = lane; j < HCAP; j += 32) {
-        hkey[j] = -1;
-        hdist[j] = kInf;
-        hst[j] = kFrontier;
+    for (int j = 4 * lane; j < HCAP; j += 128) {
+        *reinterpret_cast<int4*>(hkey + j) = make_int4(-1, -1, -1, -1);
+        if constexpr (kNarrow)
+            *reinterpret_cast<uint4*>(hdist + j) = make_uint4(~0u, ~0u, ~0u, ~0u);
+        else
+            for (int i = 0; i < 4; ++i) hdist[j + i] = kInf;
     }
     __syncwarp();
     if (lane == 0) {
@@ -684,15 +774,24 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
     }
     __syncwarp();
     int status = 0, nset = 0;
+    DT last = 0, m = 0;  // the frontier minimum at the step before the last, and at the last
     for (int step = 0; step < HCAP; ++step) {  // every step settles at least the frontier minimum
         const int nf = *fcount;
-        if (nf == 0) break;  // every reachable seed is settled
-        long long m = kInf;
+        if (nf == 0) {  // every reachable seed is settled
+            last = 0;
+            m = kInf;
+            break;
+        }
+        last = m;  // fewer than k settled seeds lie below it
+        m = kInf;
         for (int i = lane; i < nf; i += 32) m = min(m, hdist[front[i]]);
-        m = warp_min64(m);
-        int below = 0;
-        for (int i = lane; i < nset; i += 32) below += (long long)(skey[i] >> kIdxBits) < m;
-        if ((int)__reduce_add_sync(0xffffffffu, (unsigned)below) >= a.k) break;
+        m = warp_min(m);
+        if (nset >= a.k) {
+            const unsigned long long bound = (unsigned long long)m << kIdxBits;
+            int below = 0;
+            for (int i = lane; i < nset; i += 32) below += skey[i] < bound;
+            if ((int)__reduce_add_sync(0xffffffffu, (unsigned)below) >= a.k) break;
+        }
         // settle the batch: compact the frontier list in place (chunks are read
         // before the kept entries of the chunk are written, and never ahead of them)
         const int nset0 = nset;
@@ -700,20 +799,18 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
         for (int c = 0; c < nf; c += 32) {
             const int i = c + lane;
             int h = -1;
+            DT d = 0;
             bool bat = false;
             if (i < nf) {
                 h = front[i];
-                bat = hdist[h] <= m + (long long)hmin[h];
+                d = hdist[h];
+                bat = d - m <= (DT)hmin[h];
             }
             const unsigned bm = __ballot_sync(0xffffffffu, bat), km = __ballot_sync(0xffffffffu, i < nf && !bat);
             const unsigned lt = (1u << lane) - 1;
-            __syncwarp();
             if (bat) {
                 const int pos = nset + __popc(bm & lt);
-                if (pos < SCAP) {
-                    skey[pos] = ((unsigned long long)hdist[h] << kIdxBits) | (unsigned long long)hkey[h];
-                    hst[h] = kSettled;
-                }
+                if (pos < SCAP) skey[pos] = ((unsigned long long)d << kIdxBits) | (unsigned long long)hkey[h];
             } else if (i < nf) {
                 front[kept + __popc(km & lt)] = (short)h;
             }
@@ -728,18 +825,20 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
         if (lane == 0) *fcount = kept;
         __syncwarp();
         // relax the batch's links, one lane per link: the batch seeds' link counts
-        // are prefix-summed over the warp (32 seeds at a time) and each lane finds
-        // the seed owning its link by a binary search over the sums, so all the
-        // links' loads are in flight together
+        // are prefix-summed over the warp (32 seeds at a time); in a chunk of 32 links
+        // the seeds whose lists begin in it set a bit at their first link, and a lane's
+        // owner is the last seed that begins at or before its link (every batch seed
+        // has a link: it was reached through one, or is s, alone or with links), so all
+        // the links' loads are in flight together
         int st = 0;
         for (int b0 = nset0; b0 < nset; b0 += 32) {
             const int nb = min(32, nset - b0);
             int u = 0, first = 0, deg = 0;
-            long long du = 0;
+            DT du = 0;
             if (lane < nb) {
                 const unsigned long long kb = skey[b0 + lane];
                 u = (int)(kb & kIdxMask);
-                du = (long long)(kb >> kIdxBits);
+                du = (DT)(kb >> kIdxBits);
                 first = a.off[u];
                 deg = a.end_of[u] - first;
             }
@@ -749,26 +848,23 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
                 const int y = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += y;
             }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            const int total = __shfl_sync(0xffffffffu, incl, 31), excl = incl - deg;
             for (int c0 = 0; c0 < total; c0 += 32) {
-                const int e = c0 + lane;
-                // owner: the first batch lane whose inclusive sum exceeds e
-                int lo = 0, hi = nb - 1;
-#pragma unroll
-                for (int it = 0; it < 5; ++it) {
-                    const int mid = (lo + hi) >> 1;
-                    const int v = __shfl_sync(0xffffffffu, incl, mid);
-                    if (v > e) hi = mid; else lo = min(mid + 1, hi);
-                }
-                const int ow = lo;
-                const int ofirst = __shfl_sync(0xffffffffu, first, ow);
-                const int oexcl = __shfl_sync(0xffffffffu, incl - deg, ow);
-                const long long odu = __shfl_sync(0xffffffffu, du, ow);
+                const int e = c0 + lane, rel = excl - c0;
+                const bool here = lane < nb && rel >= 0 && rel < 32;
+                const unsigned starts = __reduce_or_sync(0xffffffffu, here ? 1u << rel : 0u);
+                const int before = __popc(__ballot_sync(0xffffffffu, lane < nb && rel < 0));
+                const int ow = max(before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1, 0);
+                const int le = __shfl_sync(0xffffffffu, first - excl, ow) + e;
+                const DT odu = __shfl_sync(0xffffffffu, du, ow);
                 if (e >= total || st) continue;
-                const int le = ofirst + (e - oexcl);
-                const int4 li = a.adj_i[le];
-                const long long nd = odu + a.adj_w[le];
+                const int4 li = __ldg(a.adj + le);  // neighbour, its smallest link weight, the link's weight
+                const long long nd = (long long)odu + (long long)(((unsigned long long)(unsigned)li.w << 32) | (unsigned)li.z);
                 if (nd >= kDistLimit) st |= kErrRange;
+                if (kNarrow && nd >= (long long)kInf) {  // (a pixel's distance stays below 2^31; links of many may not)
+                    st |= kRetry;
+                    continue;
+                }
                 const int t = li.x;
                 int h = slot_of(t), hs = -1;
                 for (int q = 0; q < HCAP; ++q) {
@@ -780,7 +876,7 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
                     if (c == -1) {
                         const int prev = atomicCAS(&hkey[h], -1, t);
                         if (prev == -1) {  // discovered: joins the frontier list
-                            hmin[h] = (unsigned)li.w;
+                            hmin[h] = (unsigned)li.y;
                             const int f = atomicAdd(fcount, 1);
                             if (f < FCAP)
                                 front[f] = (short)h;
@@ -801,8 +897,7 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
                     continue;
                 }
                 // a settled seed keeps its final distance: the minimum is a no-op there
-                if (hst[hs] == kFrontier)
-                    atomicMin(reinterpret_cast<unsigned long long*>(&hdist[hs]), (unsigned long long)nd);
+                atomic_min_shared(&hdist[hs], (DT)nd);
             }
         }
         __syncwarp();
@@ -810,16 +905,24 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
         if (status) break;
     }
     if (!status) {
-        int N = 32;
-        while (N < nset) N <<= 1;
-        if (N > SCAP) {
-            status = kRetry;
-        } else {
-            for (int j = nset + lane; j < N; j += 32) skey[j] = kNone;
-            __syncwarp();
-            warp_bitonic_sort(skey, N);
-            cnt_out = min(nset, a.k);
+        const int want = min(nset, a.k);
+        cnt_out = want;
+        const int room = want <= 32 ? 32 : want <= 64 ? 64 : want <= 128 ? 128 : 256;  // the sort's width
+        int n = nset;
+        if (n > room) {
+            // every settled key of the list is below 2^40, and of those below m at least k
+            const long long hi = (long long)m < kDistLimit ? (long long)m : kDistLimit - 1;
+            warp_select(skey, n, want, (long long)last, hi);
+            n = want;
         }
+        if (room == 32)
+            warp_sort<1>(skey, n);
+        else if (room == 64)
+            warp_sort<2>(skey, n);
+        else if (room == 128)
+            warp_sort<4>(skey, n);
+        else
+            warp_sort<8>(skey, n);
     }
     return status & kErrRange ? kErrRange : status;
 }
@@ -933,7 +1036,7 @@ __global__ void __launch_bounds__(kThreads) epic_solve_kernel(KnnArgs a)
 template <int HCAP, int FCAP, int SCAP>
 __global__ void __launch_bounds__(kFastWarps * 32) epic_knn_fit_kernel(KnnArgs a)
 {
-    using Lay = KnnLayout<HCAP, FCAP, SCAP>;
+    using Lay = KnnLayout<unsigned, HCAP, FCAP, SCAP>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int idx = a.begin + blockIdx.x * kFastWarps + wid;
@@ -941,7 +1044,7 @@ __global__ void __launch_bounds__(kFastWarps * 32) epic_knn_fit_kernel(KnnArgs a
     const int s = a.list[idx];
     unsigned char* base = smem + (size_t)wid * Lay::bytes;
     int cnt = 0;
-    const int st = knn_search<HCAP, FCAP, SCAP>(a, s, base, cnt);
+    const int st = knn_search<unsigned, HCAP, FCAP, SCAP>(a, s, base, cnt);
     if (st == kRetry) {
         if (lane == 0) a.retry_list[atomicAdd(a.retry_count, 1)] = idx;
         return;
@@ -957,7 +1060,7 @@ __global__ void __launch_bounds__(kFastWarps * 32) epic_knn_fit_kernel(KnnArgs a
 // warp per block.
 __global__ void __launch_bounds__(32) epic_knn_retry_kernel(KnnArgs a)
 {
-    using Lay = KnnLayout<kBigH, kBigF, kBigS>;
+    using Lay = RetryLayout;
     extern __shared__ __align__(16) unsigned char smem[];
     const int total = *a.retry_count;
     for (int i = blockIdx.x; i < total; i += gridDim.x) {
@@ -965,7 +1068,7 @@ __global__ void __launch_bounds__(32) epic_knn_retry_kernel(KnnArgs a)
         if (idx < a.begin) continue;  // of an earlier launch
         const int s = a.list[idx];
         int cnt = 0;
-        const int st = knn_search<kBigH, kBigF, kBigS>(a, s, smem, cnt);
+        const int st = knn_search<long long, kBigH, kBigF, kBigS>(a, s, smem, cnt);
         if (st) {
             if ((threadIdx.x & 31) == 0) atomicOr(a.err, st == kRetry ? kErrFrontier : st);
             continue;
@@ -1174,8 +1277,7 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         a.off = off;
         a.end_of = cur;
         a.minin = minin;
-        a.adj_i = adj_i;
-        a.adj_w = adj_w;
+        a.adj = adj_i;
         a.models = models;
         a.err = err;
         a.retry_count = retry_count;
@@ -1192,9 +1294,8 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         a.min_spread2 = p->min_spread * p->min_spread;
         const bool small = p->k <= kSmallK;
         auto fast = small ? epic_knn_fit_kernel<384, 256, 256> : epic_knn_fit_kernel<1024, 512, 512>;
-        const size_t smem_fast =
-            (small ? KnnLayout<384, 256, 256>::bytes : KnnLayout<1024, 512, 512>::bytes) * kFastWarps;
-        const size_t smem_big = KnnLayout<kBigH, kBigF, kBigS>::bytes;
+        const size_t smem_fast = (small ? SmallLayout::bytes : LargeLayout::bytes) * kFastWarps;
+        const size_t smem_big = RetryLayout::bytes;
         if (cudaFuncSetAttribute(fast, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fast) != cudaSuccess ||
             cudaFuncSetAttribute(epic_knn_retry_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_big) !=
                 cudaSuccess)
@@ -1211,7 +1312,7 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         a.list_count = list_count;
         a.n_weights = n_weights;
         a.weights = reinterpret_cast<const float2*>(cost);
-        epic_link_meta_kernel<<<pt_grid, kThreads, 0, stream>>>(a, adj_t, adj_i, list, list_count);
+        epic_link_meta_kernel<<<pt_grid, kThreads, 0, stream>>>(a, adj_t, adj_w, adj_i, list, list_count);
         a.sums = reinterpret_cast<double*>(adj_t);
         const long long holders = std::min<long long>(n, (long long)W * H);
         const long long room = (long long)((L.adj_w - L.adj_t) / (12 * sizeof(double)));
