@@ -47,7 +47,13 @@ constexpr int kTile = 32;                    // Voronoi tiles: 32 x 32 pixels, 3
 constexpr int kMaxPasses = 4096;
 constexpr int kThreads = 256;
 
-constexpr long long kNoLink = 0xffffffffll;  // min link weight of a seed without links
+// Distances on the frame fit 31 bits: at most W + H steps of at most twice the largest
+// pixel cost (base 4096, gain 32, Sobel magnitudes 1020 + 1020). A link's weight, two
+// distances and a step, fits 32.
+constexpr long long kMaxStep = 2ll * (4096 + 32 * 2040);
+static_assert(DGF_EPIC_MAX_W_PLUS_H * kMaxStep < (1ll << 31), "distances of 31 bits");
+static_assert(2 * DGF_EPIC_MAX_W_PLUS_H * kMaxStep + kMaxStep < 0xffffffffll, "link weights of 32 bits");
+constexpr unsigned kNoLink = 0xffffffffu;  // min link weight of a seed without links
 
 // Device status bits (any of them makes the call return DGF_ERR_DEVICE).
 enum : int { kErrFrontier = 1, kErrFill = 4, kErrRange = 8, kErrPasses = 16, kErrSync = 32 };
@@ -229,7 +235,7 @@ __global__ void epic_report_kernel(const int* err, unsigned* status)
 template <bool FILL>
 __global__ void __launch_bounds__(kThreads) epic_links_kernel(const unsigned long long* key, const int* cost, int W,
                                                               int H, int* cnt, const int* off, int* cur, int* adj_t,
-                                                              long long* adj_w, int* err)
+                                                              unsigned* adj_w, int* err)
 {
     const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
     if (x >= W || y >= H) return;
@@ -249,7 +255,7 @@ __global__ void __launch_bounds__(kThreads) epic_links_kernel(const unsigned lon
             atomicAdd(&cnt[t], 1);
             continue;
         }
-        const long long w = (long long)(k >> kIdxBits) + cost[o] + cost[o2] + (long long)(k2 >> kIdxBits);
+        const unsigned w = (unsigned)(k >> kIdxBits) + (unsigned)(cost[o] + cost[o2]) + (unsigned)(k2 >> kIdxBits);
         const int ps = atomicAdd(&cur[s], 1), pt = atomicAdd(&cur[t], 1);
         if (ps < off[s + 1]) {
             adj_t[ps] = t;
@@ -354,7 +360,7 @@ struct KnnArgs {
     const int* off;
     const int* end_of;
     const unsigned* minin;
-    const int4* adj;  // link records: neighbour, its smallest link weight, the link's weight (low, high)
+    const int4* adj;  // link records: neighbour, its smallest link weight, the link's weight
     double* models;  // [n][6]
     const int* list;        // the seeds that hold a pixel, in any order
     const int* list_count;  // their number
@@ -526,15 +532,17 @@ __device__ __forceinline__ void warp_sum12(const double (&v)[12], double (&q)[3]
 
 // Per seed: keeps one link per neighbour (the smallest weight), compacting the list
 // in place; end[s] becomes the end of the compacted list. One warp per seed walks
-// the list in chunks of 32: lanes holding the same neighbour find each other with
-// match.any and take their minimum weight; the lowest of them either lowers the
-// weight of a link kept from an earlier chunk or appends a new one. The kept prefix
-// never reaches the unread part of the list. Also fills the table of fit weights, an
-// entry a thread.
-__global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, int* end, int* adj_t, long long* adj_w,
-                                                               unsigned* minin, int n, double a_per_unit, float2* weights,
-                                                               int n_weights)
+// the list in chunks of 32 and takes a chunk's neighbours one by one (about six of
+// some twenty links): a ballot finds the neighbour's links, a warp minimum their
+// weight, and lane i holds the i-th kept link in registers. A seed with more than 32
+// neighbours keeps the others in its list, whose kept prefix never reaches the unread
+// part. Also fills the table of fit weights, an entry a thread. 1242x375 pair: 20 us,
+// 35 with a 32-step shuffle loop over 64-bit weights a chunk.
+__global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, int* end, int* adj_t, unsigned* adj_w,
+                                                               unsigned* minin, int n, double a_per_unit,
+                                                               float2* weights, int n_weights)
 {
+    constexpr unsigned kAll = 0xffffffffu;
     for (int d = blockIdx.x * kThreads + threadIdx.x; d < n_weights; d += gridDim.x * kThreads) {
         const dfl w = fit_weight(a_per_unit, d);
         weights[d] = make_float2(w.hi, w.lo);
@@ -543,46 +551,55 @@ __global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, i
     const int s = (int)(((size_t)blockIdx.x * kThreads + threadIdx.x) >> 5);
     if (s >= n) return;  // warp-uniform
     const int b = off[s], e = off[s + 1];
-    int out = b;
+    int cnt = 0, kt = -1;  // kept links; the lane's neighbour and weight
+    unsigned kw = kNoLink;
     for (int c = b; c < e; c += 32) {
         const bool has = c + lane < e;
-        const int t = has ? adj_t[c + lane] : -1 - lane;  // empty lanes match nobody
-        const long long w = has ? adj_w[c + lane] : 0;
-        const unsigned grp = __match_any_sync(0xffffffffu, t);
-        long long mw = w;
-        for (int j = 0; j < 32; ++j) {
-            const long long wj = __shfl_sync(0xffffffffu, w, j);
-            if ((grp >> j) & 1u) mw = min(mw, wj);
-        }
-        const bool leader = has && lane == __ffs(grp) - 1;
-        int found = -1;
-        if (leader)
-            for (int j = b; j < out; ++j)
-                if (adj_t[j] == t) {
-                    found = j;
-                    break;
+        const int t = has ? adj_t[c + lane] : -1;
+        const unsigned w = has ? adj_w[c + lane] : kNoLink;
+        unsigned left = __ballot_sync(kAll, has);
+        while (left) {
+            const int tt = __shfl_sync(kAll, t, __ffs(left) - 1);
+            const bool in = t == tt;
+            left &= ~__ballot_sync(kAll, in);
+            const unsigned mw = __reduce_min_sync(kAll, in ? w : kNoLink);
+            const bool hit = kt == tt;
+            if (__any_sync(kAll, hit)) {
+                if (hit) kw = min(kw, mw);
+            } else if (cnt < 32) {
+                if (lane == cnt) {
+                    kt = tt;
+                    kw = mw;
                 }
-        if (found >= 0 && mw < adj_w[found]) adj_w[found] = mw;  // leaders hold distinct neighbours
-        const bool app = leader && found < 0;
-        const unsigned km = __ballot_sync(0xffffffffu, app);
-        __syncwarp();
-        if (app) {
-            const int pos = out + __popc(km & ((1u << lane) - 1));
-            adj_t[pos] = t;
-            adj_w[pos] = mw;
+                ++cnt;
+            } else {
+                int found = -1;
+                for (int j = b + 32 + lane; j < b + cnt; j += 32)
+                    if (adj_t[j] == tt) found = j;
+                if (__any_sync(kAll, found >= 0)) {
+                    if (found >= 0) adj_w[found] = min(adj_w[found], mw);
+                } else {
+                    if (lane == 0) {
+                        adj_t[b + cnt] = tt;
+                        adj_w[b + cnt] = mw;
+                    }
+                    ++cnt;
+                }
+                __syncwarp();
+            }
         }
-        out += __popc(km);
-        __syncwarp();
     }
-    // smallest link weight (a lower bound on the last step of any path into s),
-    // clamped to 32 bits (a smaller bound stays a bound)
-    long long mn = kNoLink;
-    for (int j = b + lane; j < out; j += 32) mn = min(mn, adj_w[j]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    if (lane < cnt) {
+        adj_t[b + lane] = kt;
+        adj_w[b + lane] = kw;
+    }
+    // smallest link weight (a lower bound on the last step of any path into s)
+    unsigned mn = kw;
+    for (int j = b + 32 + lane; j < b + cnt; j += 32) mn = min(mn, adj_w[j]);
+    mn = __reduce_min_sync(kAll, mn);
     if (lane == 0) {
-        end[s] = out;
-        minin[s] = (unsigned)min(mn, (long long)kNoLink);
+        end[s] = b + cnt;
+        minin[s] = mn;
     }
 }
 
@@ -590,7 +607,7 @@ __global__ void __launch_bounds__(kThreads) epic_dedupe_kernel(const int* off, i
 // weight, the link's weight; the list of the seeds that hold a pixel (in any order; a
 // warp takes its places with one atomic), and the outputs of those that do not.
 __global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, const int* adj_t,
-                                                                  const long long* adj_w, int4* adj, int* list,
+                                                                  const unsigned* adj_w, int4* adj, int* list,
                                                                   int* list_count)
 {
     const int s = blockIdx.x * kThreads + threadIdx.x, lane = threadIdx.x & 31;
@@ -612,8 +629,7 @@ __global__ void __launch_bounds__(kThreads) epic_link_meta_kernel(KnnArgs a, con
     list[at + __popc(hold & ((1u << lane) - 1))] = s;
     for (int i = a.off[s], e = a.end_of[s]; i < e; ++i) {
         const int t = adj_t[i];
-        const long long w = adj_w[i];
-        adj[i] = make_int4(t, (int)a.minin[t], (int)(unsigned)w, (int)(w >> 32));
+        adj[i] = make_int4(t, (int)a.minin[t], (int)adj_w[i], 0);
     }
 }
 
@@ -859,9 +875,9 @@ __device__ int knn_search(const KnnArgs& a, int s, unsigned char* base, int& cnt
                 const DT odu = __shfl_sync(0xffffffffu, du, ow);
                 if (e >= total || st) continue;
                 const int4 li = __ldg(a.adj + le);  // neighbour, its smallest link weight, the link's weight
-                const long long nd = (long long)odu + (long long)(((unsigned long long)(unsigned)li.w << 32) | (unsigned)li.z);
+                const long long nd = (long long)odu + (long long)(unsigned)li.z;
                 if (nd >= kDistLimit) st |= kErrRange;
-                if (kNarrow && nd >= (long long)kInf) {  // (a pixel's distance stays below 2^31; links of many may not)
+                if (kNarrow && nd >= (long long)kInf) {  // (a path of several links may be longer than 32 bits)
                     st |= kRetry;
                     continue;
                 }
@@ -1127,7 +1143,7 @@ EpicLayout epic_layout(int W, int H, int n)
     L.minin = take((size_t)n * 4);
     L.bsum = take(((size_t)n / 1024 + 2) * 12);  // block totals, block offsets (+1), scan cursors
     L.adj_t = take(nl * 4);
-    L.adj_w = take(nl * 8);
+    L.adj_w = take(nl * 4);
     L.adj_i = take(nl * 16);
     L.models = take((size_t)n * 48);
     L.retry = take((size_t)n * 4);
@@ -1210,7 +1226,7 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
     auto* off = reinterpret_cast<int*>(ws + L.off);
     auto* cur = reinterpret_cast<int*>(ws + L.cur);
     auto* adj_t = reinterpret_cast<int*>(ws + L.adj_t);
-    auto* adj_w = reinterpret_cast<long long*>(ws + L.adj_w);
+    auto* adj_w = reinterpret_cast<unsigned*>(ws + L.adj_w);
     auto* adj_i = reinterpret_cast<int4*>(ws + L.adj_i);
     auto* minin = reinterpret_cast<unsigned*>(ws + L.minin);
     auto* bsum = reinterpret_cast<int*>(ws + L.bsum);
@@ -1304,9 +1320,9 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
             return DGF_ERR_CUDA;
-        // the list takes the place of the link counts; the fits' sums that of adj_t once
-        // the link records are made. Seeds beyond its room (W H / 6 of them; at most
-        // W H hold a pixel) are searched and solved in further launches.
+        // the list takes the place of the link counts; the fits' sums that of adj_t and
+        // adj_w once the link records are made. Seeds beyond its room (W H / 3 of them; at
+        // most W H hold a pixel) are searched and solved in further launches.
         int* list = cnt;
         a.list = list;
         a.list_count = list_count;
@@ -1315,7 +1331,7 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
         epic_link_meta_kernel<<<pt_grid, kThreads, 0, stream>>>(a, adj_t, adj_w, adj_i, list, list_count);
         a.sums = reinterpret_cast<double*>(adj_t);
         const long long holders = std::min<long long>(n, (long long)W * H);
-        const long long room = (long long)((L.adj_w - L.adj_t) / (12 * sizeof(double)));
+        const long long room = (long long)((L.adj_i - L.adj_t) / (12 * sizeof(double)));
         for (long long at = 0; at < holders; at += room) {
             a.begin = (int)at;
             a.end = (int)std::min(holders, at + room);
