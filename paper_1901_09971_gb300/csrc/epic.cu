@@ -43,7 +43,7 @@ constexpr unsigned long long kNone = ~0ull;
 constexpr int kIdxBits = 24;
 constexpr unsigned long long kIdxMask = (1ull << kIdxBits) - 1;
 constexpr long long kDistLimit = 1ll << 40;  // the distance field of a packed key
-constexpr int kTile = 32;                    // Voronoi tiles: 32 x 32 pixels, 32 x 8 threads
+constexpr int kTile = 32, kBand = 4;         // Voronoi tiles: 32 x 32 pixels, 32 x 8 threads, four rows a warp
 constexpr int kMaxPasses = 4096;
 constexpr int kThreads = 256;
 
@@ -103,78 +103,132 @@ __global__ void __launch_bounds__(kThreads) epic_seed_owner_kernel(const unsigne
     if (o >= 0 && key[o] != (unsigned long long)i) seed_pix[i] = -1;
 }
 
-__device__ __forceinline__ void relax(unsigned long long& best, unsigned long long kn, int w)
+// Labelling keys in registers: an unreached pixel holds kFar, from which no step
+// improves anything (real keys lie below kReal: a distance of 31 bits and 24 of index),
+// and an edge to a pixel outside the frame weighs kWall, which takes any key past them.
+constexpr unsigned long long kFar = 1ull << 63, kReal = 1ull << 55;
+constexpr unsigned kWall = 0xffffffffu;
+__device__ __forceinline__ void relax(unsigned long long& best, unsigned long long kn, unsigned w)
 {
-    if (kn != kNone) best = min(best, kn + ((unsigned long long)w << kIdxBits));
+    best = min(best, kn + (unsigned long long)w * (1ull << kIdxBits));
 }
 
-// One relaxation pass over the 32 x 32 tile at (x0, y0): the tile and a one-pixel
-// halo in shared memory, Jacobi min-plus sweeps until the tile is stable, improved
-// keys written back with atomicMin; counts the tile in changed[pass] if any key
-// improved. Called by every thread of the block.
+// Rows of a tile that other warps read: the first and the last of each warp's band.
+// Plain 8-byte shared accesses (never torn), volatile so that every sweep reads anew.
+struct VoronoiEdges {
+    volatile unsigned long long top[kTile / kBand][kTile], bot[kTile / kBand][kTile];
+};
+
+// One relaxation pass over the 32 x 32 tile at (x0, y0): a warp owns a band of four rows
+// and a lane a column of it, keys and edge weights in registers, the neighbouring
+// tiles' border keys (halo) fixed for the pass. A sweep relaxes each pixel from its
+// left and right neighbours (shuffles), then down and up the band (a path runs
+// through the whole band in one sweep), the bands' border rows passing through shared
+// memory. The min-plus fixed point does not depend on the order, so warps sweep
+// without waiting for one another (a stale border row is a valid upper bound) and only
+// every third sweep is closed by a barrier before and a vote after it: once it changes
+// nothing, every pixel was checked against final neighbours. Improved keys are
+// written back (the tile's pixels are written by nobody else); counts the tile in
+// changed[pass] if any key improved. Called by every thread of the block.
+// What bounds it is the latency of one sweep times the longest path inside a tile
+// (shortest paths through seedless areas wind for 50 pixels and more). With a thread
+// per four scattered pixels, all keys in shared memory and two barriers a sweep, a
+// sweep took about 1,250 cycles and moved a path one pixel: 227 us of labelling on the
+// 1242x375 pair, 129 us now.
 __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long* key, int W, int H, int* changed,
-                                             int pass, int x0, int y0)
+                                             int pass, int x0, int y0, VoronoiEdges& E)
 {
-    __shared__ unsigned long long sk[kTile + 2][kTile + 2];
-    __shared__ int sc[kTile + 2][kTile + 2];
-    const int tid = threadIdx.y * 32 + threadIdx.x;
-    for (int e = tid; e < (kTile + 2) * (kTile + 2); e += kThreads) {
-        const int ly = e / (kTile + 2), lx = e - ly * (kTile + 2);
-        const int gx = x0 + lx - 1, gy = y0 + ly - 1;
-        unsigned long long k = kNone;
-        int c = 0;
-        if (gx >= 0 && gx < W && gy >= 0 && gy < H) {
-            const size_t o = (size_t)gy * W + gx;
-            // halo keys belong to other tiles, which may lower them concurrently;
-            // any value read is a valid upper bound
-            k = *reinterpret_cast<const volatile unsigned long long*>(key + o);
-            c = cost[o];
+    const int lane = threadIdx.x, w = threadIdx.y;
+    const int x = x0 + lane, yb = y0 + kBand * w;
+    const bool xin = x < W;
+    auto load_key = [&](int px, int py) {
+        if (px < 0 || px >= W || py < 0 || py >= H) return kFar;
+        // halo keys belong to other tiles, which may lower them concurrently; any
+        // value read is a valid upper bound
+        return min(*reinterpret_cast<const volatile unsigned long long*>(key + (size_t)py * W + px), kFar);
+    };
+    auto load_cost = [&](int px, int py) {
+        return px >= 0 && px < W && py >= 0 && py < H ? (unsigned)cost[(size_t)py * W + px] : kWall;
+    };
+    auto edge = [](unsigned a, unsigned b) { return a == kWall || b == kWall ? kWall : a + b; };
+    unsigned long long k[kBand], orig[kBand], side[kBand];  // side: the halo beside lanes 0 and 31
+    unsigned wl[kBand], wr[kBand], wv[kBand + 1];
+    {
+        unsigned c[kBand + 2];
+        const int xs = lane == 0 ? x - 1 : x + 1;  // used by lanes 0 and 31
+        const bool outer = lane == 0 || lane == 31;
+#pragma unroll
+        for (int r = 0; r < kBand; ++r) {
+            orig[r] = k[r] = load_key(x, yb + r);
+            side[r] = outer ? load_key(xs, yb + r) : kFar;
         }
-        sk[ly][lx] = k;
-        sc[ly][lx] = c;
+#pragma unroll
+        for (int r = 0; r < kBand + 2; ++r) c[r] = load_cost(x, yb + r - 1);
+#pragma unroll
+        for (int r = 0; r < kBand; ++r) {
+            const unsigned cs = outer ? load_cost(xs, yb + r) : 0u;
+            unsigned cl = __shfl_up_sync(0xffffffffu, c[r + 1], 1), cr = __shfl_down_sync(0xffffffffu, c[r + 1], 1);
+            if (lane == 0) cl = cs;
+            if (lane == 31) cr = cs;
+            wl[r] = edge(c[r + 1], cl);
+            wr[r] = edge(c[r + 1], cr);
+        }
+#pragma unroll
+        for (int r = 0; r <= kBand; ++r) wv[r] = edge(c[r], c[r + 1]);
     }
+    // the halo rows above and below the tile, or the neighbouring bands' border rows
+    const bool first = w == 0, last = w == kTile / kBand - 1;
+    const unsigned long long above = first ? load_key(x, yb - 1) : kFar, below = last ? load_key(x, yb + kBand) : kFar;
+    E.top[w][lane] = k[0];
+    E.bot[w][lane] = k[kBand - 1];
     __syncthreads();
-    const int lx = threadIdx.x + 1;
-    const bool xin = x0 + threadIdx.x < W;
-    unsigned long long orig[kTile / 8];
-#pragma unroll
-    for (int r = 0; r < kTile / 8; ++r) orig[r] = sk[threadIdx.y + 8 * r + 1][lx];
-    // Jacobi sweeps with the halo fixed; a sweep extends every shortest path by one
-    // step, so the tile is stable after at most kTile^2 sweeps
-    for (int it = 0; it <= kTile * kTile; ++it) {
-        unsigned long long nk[kTile / 8];
+    auto sweep = [&]() {
+        const unsigned long long up = first ? above : E.bot[w - 1][lane], dn = last ? below : E.top[w + 1][lane];
         bool ch = false;
+        unsigned long long b[kBand];
 #pragma unroll
-        for (int r = 0; r < kTile / 8; ++r) {
-            const int ly = threadIdx.y + 8 * r + 1;
-            unsigned long long best = sk[ly][lx];
-            if (xin && y0 + ly - 1 < H) {
-                const int c = sc[ly][lx];
-                relax(best, sk[ly][lx - 1], sc[ly][lx - 1] + c);
-                relax(best, sk[ly][lx + 1], sc[ly][lx + 1] + c);
-                relax(best, sk[ly - 1][lx], sc[ly - 1][lx] + c);
-                relax(best, sk[ly + 1][lx], sc[ly + 1][lx] + c);
-                ch |= best < sk[ly][lx];
-            }
-            nk[r] = best;
+        for (int r = 0; r < kBand; ++r) {
+            unsigned long long l = __shfl_up_sync(0xffffffffu, k[r], 1), t = __shfl_down_sync(0xffffffffu, k[r], 1);
+            if (lane == 0) l = side[r];
+            if (lane == 31) t = side[r];
+            b[r] = k[r];
+            relax(b[r], l, wl[r]);
+            relax(b[r], t, wr[r]);
         }
-        __syncthreads();
+        relax(b[0], up, wv[0]);
 #pragma unroll
-        for (int r = 0; r < kTile / 8; ++r) sk[threadIdx.y + 8 * r + 1][lx] = nk[r];
-        if (!__syncthreads_or(ch)) break;
+        for (int r = 1; r < kBand; ++r) relax(b[r], b[r - 1], wv[r]);
+        relax(b[kBand - 1], dn, wv[kBand]);
+#pragma unroll
+        for (int r = kBand - 2; r >= 0; --r) relax(b[r], b[r + 1], wv[r + 1]);
+#pragma unroll
+        for (int r = 0; r < kBand; ++r) {
+            ch |= b[r] < k[r];
+            k[r] = b[r];
+        }
+        E.top[w][lane] = k[0];
+        E.bot[w][lane] = k[kBand - 1];
+        return ch;
+    };
+    // a sweep between barriers extends every shortest path by at least one step, so the
+    // tile is stable after at most kTile^2 rounds
+    for (int it = 0; it <= kTile * kTile; ++it) {
+        if (it) {
+            sweep();
+            sweep();
+            __syncthreads();
+        }
+        if (!__syncthreads_or(sweep())) break;
     }
     bool improved = false;
 #pragma unroll
-    for (int r = 0; r < kTile / 8; ++r) {
-        const int ly = threadIdx.y + 8 * r + 1;
-        const unsigned long long k = sk[ly][lx];
-        if (k < orig[r]) {
-            atomicMin(&key[(size_t)(y0 + ly - 1) * W + x0 + lx - 1], k);
+    for (int r = 0; r < kBand; ++r)
+        if (k[r] < min(orig[r], kReal) && xin && yb + r < H) {
+            key[(size_t)(yb + r) * W + x] = k[r];
             improved = true;
         }
-    }
-    if (__syncthreads_or(improved) && tid == 0) atomicAdd(&changed[pass], 1);
-    __syncthreads();  // the next tile reuses sk and sc
+    // (also keeps the next tile's border rows behind this tile's last sweep)
+    if (__syncthreads_or(improved) && lane == 0 && w == 0) atomicAdd(&changed[pass], 1);
 }
 
 // Barrier of all blocks of a cooperative launch (all co-resident): arrivals on a
@@ -207,14 +261,15 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target)
 // stop at the first that changed nothing (every block reads the same count after
 // the barrier) or after kMaxPasses, which is recorded as a failure; so is a barrier
 // that gave up. No host round trip between passes.
-__global__ void __launch_bounds__(kThreads) epic_voronoi_kernel(const int* cost, unsigned long long* key, int W, int H,
+__global__ void __launch_bounds__(kThreads, 4) epic_voronoi_kernel(const int* cost, unsigned long long* key, int W, int H,
                                                                 int* changed, unsigned* sync_count, int* err)
 {
+    __shared__ VoronoiEdges edges;
     const int tiles_x = (W + kTile - 1) / kTile, n_tiles = tiles_x * ((H + kTile - 1) / kTile);
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0;
     for (int pass = 0; pass < kMaxPasses; ++pass) {
         for (int t = blockIdx.x; t < n_tiles; t += gridDim.x)
-            voronoi_tile(cost, key, W, H, changed, pass, (t % tiles_x) * kTile, (t / tiles_x) * kTile);
+            voronoi_tile(cost, key, W, H, changed, pass, (t % tiles_x) * kTile, (t / tiles_x) * kTile, edges);
         if (!grid_barrier(sync_count, (unsigned)(pass + 1) * gridDim.x)) {
             if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(err, kErrSync);
             return;
