@@ -704,8 +704,10 @@ __device__ __forceinline__ void atomic_min_shared(unsigned* p, unsigned v) { ato
 
 // Ascending sort of the first n <= 32 P keys of a shared array by one warp: P keys a
 // lane in registers (lane l holds elements P l .. P l + P - 1), a bitonic network whose
-// strides below P stay in the lane and whose others are shuffles. Slots past n are
-// filled with the largest key and not written back.
+// strides below P stay in the lane and whose others are shuffles. The shuffle stages
+// are a loop: unrolled, they are some 700 instructions that each search runs once,
+// and fetching them stalled the warps. Slots past n are filled with the largest key and
+// not written back.
 template <int P>
 __device__ __forceinline__ void warp_sort(unsigned long long* key, int n)
 {
@@ -713,31 +715,39 @@ __device__ __forceinline__ void warp_sort(unsigned long long* key, int n)
     unsigned long long v[P];
 #pragma unroll
     for (int i = 0; i < P; ++i) v[i] = lane + 32 * i < n ? key[lane + 32 * i] : kNone;  // any order will do
+    auto exchange = [&](int i, int j, bool asc) {  // elements i < j of the lane
+        const unsigned long long x = v[i], y = v[j];
+        const bool keep = (x < y) == asc;
+        v[i] = keep ? x : y;
+        v[j] = keep ? y : x;
+    };
+    // sorted runs of P, ascending in even lanes
 #pragma unroll
-    for (int size = 2; size <= 32 * P; size <<= 1)
+    for (int size = 2; size <= P; size <<= 1)
 #pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            if (stride >= P) {
-                // element e's partner e ^ stride is element i of lane ^ (stride / P)
-                const int o = stride / P;
-                const bool low = (lane & o) == 0, asc = size < 32 * P ? ((lane * P) & size) == 0 : true;
+        for (int stride = size >> 1; stride > 0; stride >>= 1)
 #pragma unroll
-                for (int i = 0; i < P; ++i) {
-                    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v[i], o);
-                    v[i] = (v[i] < w) == (low == asc) ? v[i] : w;
-                }
-            } else {
+            for (int i = 0; i < P; ++i)
+                if (!(i & stride)) exchange(i, i ^ stride, size < P ? (i & size) == 0 : (lane & 1) == 0);
+    // merges of runs of `lanes` / 2 lanes
+#pragma unroll 1
+    for (int lanes = 2; lanes <= 32; lanes <<= 1) {
+        const bool asc = (lane & lanes) == 0;  // (lanes = 32: all ascending)
+#pragma unroll 1
+        for (int o = lanes >> 1; o > 0; o >>= 1) {
+            const bool low = (lane & o) == 0;
 #pragma unroll
-                for (int i = 0; i < P; ++i) {
-                    if (i & stride) continue;
-                    const bool asc = size < P ? (i & size) == 0 : size < 32 * P ? ((lane * P) & size) == 0 : true;
-                    const unsigned long long x = v[i], y = v[i ^ stride];
-                    const bool keep = (x < y) == asc;
-                    v[i] = keep ? x : y;
-                    v[i ^ stride] = keep ? y : x;
-                }
+            for (int i = 0; i < P; ++i) {
+                const unsigned long long w = __shfl_xor_sync(0xffffffffu, v[i], o);
+                v[i] = (v[i] < w) == (low == asc) ? v[i] : w;
             }
         }
+#pragma unroll
+        for (int stride = P >> 1; stride > 0; stride >>= 1)
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+                if (!(i & stride)) exchange(i, i ^ stride, asc);
+    }
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < P; ++i)
@@ -1017,6 +1027,7 @@ __device__ void knn_fit_sums(const KnnArgs& a, int idx, int s, int cnt, const un
     dfl acc[12];
 #pragma unroll
     for (int i = 0; i < 12; ++i) acc[i] = {0.f, 0.f};
+#pragma unroll 1
     for (int j = lane; j < cnt; j += 32) {
         const int t = (int)(key[j] & kIdxMask);
         const long long d = (long long)(key[j] >> kIdxBits);
@@ -1055,14 +1066,19 @@ __device__ void knn_fit_sums(const KnnArgs& a, int idx, int s, int cnt, const un
     row[2] = lane == 8 && cnt < 3 ? -tot[2] : tot[2];  // sum w > 0: a negative one marks fewer than 3 neighbours
 }
 
+// One-warp blocks: an SM's FP64 pipe takes 16 cycles a warp instruction, so eight warps
+// of a block on one SM while others idle took 20 us for 1,953 seeds (12 us with
+// one-warp blocks; 50,676 seeds 37 and 26 us).
+constexpr int kSolveThreads = 32;
+
 // Solves the fits of this launch's seeds from their sums, a thread a seed. The
 // solve is about 250 FP64 operations (a dozen divisions and square roots); GB300
 // issues an FP64 instruction of one lane no faster than one of 32, so on lane 0 of
 // each search's warp the solves kept the search kernel's FP64 pipe busy 58% of its
 // time. 1242x375 pair, 50,676 matches, k = 128: a call 1,761 -> 1,301 us.
-__global__ void __launch_bounds__(kThreads) epic_solve_kernel(KnnArgs a)
+__global__ void __launch_bounds__(kSolveThreads) epic_solve_kernel(KnnArgs a)
 {
-    const int idx = a.begin + blockIdx.x * kThreads + threadIdx.x;
+    const int idx = a.begin + blockIdx.x * kSolveThreads + threadIdx.x;
     if (idx >= min(a.end, *a.list_count)) return;
     const int s = a.list[idx];
     const double2* row = reinterpret_cast<const double2*>(a.sums + 12 * (size_t)(idx - a.begin));
@@ -1393,7 +1409,7 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
             const int m = a.end - a.begin;
             fast<<<(unsigned)((m + kFastWarps - 1) / kFastWarps), kFastWarps * 32, smem_fast, stream>>>(a);
             epic_knn_retry_kernel<<<(unsigned)sms, 32, smem_big, stream>>>(a);
-            epic_solve_kernel<<<(unsigned)((m + kThreads - 1) / kThreads), kThreads, 0, stream>>>(a);
+            epic_solve_kernel<<<(unsigned)((m + kSolveThreads - 1) / kSolveThreads), kSolveThreads, 0, stream>>>(a);
         }
     }
     epic_dense_kernel<<<pix_grid, pix_block, 0, stream>>>(key, models, p2, W, H, reinterpret_cast<float2*>(dense),
