@@ -103,14 +103,20 @@ __global__ void __launch_bounds__(kThreads) epic_seed_owner_kernel(const unsigne
     if (o >= 0 && key[o] != (unsigned long long)i) seed_pix[i] = -1;
 }
 
-// Labelling keys in registers: an unreached pixel holds kFar, from which no step
-// improves anything (real keys lie below kReal: a distance of 31 bits and 24 of index),
-// and an edge to a pixel outside the frame weighs kWall, which takes any key past them.
-constexpr unsigned long long kFar = 1ull << 63, kReal = 1ull << 55;
-constexpr unsigned kWall = 0xffffffffu;
+// Labelling keys in registers and shared memory: distance (31 bits) in the high word, seed
+// in the low one, so a step adds its weight to one word. An unreached pixel holds kFar,
+// from which no step improves anything. Pixels outside the frame hold 0, which nothing
+// improves, and steps from them weigh kWall, which ends at kFar: no improvement either.
+constexpr unsigned kWall = 0xc0000000u;
+constexpr unsigned long long kFar = (unsigned long long)kWall << 32;
+static_assert(kWall + kMaxStep < (1ll << 32), "a step from an unreached pixel stays in 32 bits");
+__device__ __forceinline__ unsigned long long step_from(unsigned long long kn, unsigned w)
+{
+    return ((unsigned long long)((unsigned)(kn >> 32) + w) << 32) | (unsigned)kn;
+}
 __device__ __forceinline__ void relax(unsigned long long& best, unsigned long long kn, unsigned w)
 {
-    best = min(best, kn + (unsigned long long)w * (1ull << kIdxBits));
+    best = min(best, step_from(kn, w));
 }
 
 // Rows of a tile that other warps read: the first and the last of each warp's band.
@@ -134,25 +140,26 @@ struct VoronoiEdges {
 // (shortest paths through seedless areas wind for 50 pixels and more). With a thread
 // per four scattered pixels, all keys in shared memory and two barriers a sweep, a
 // sweep took about 1,250 cycles and moved a path one pixel: 227 us of labelling on the
-// 1242x375 pair, 129 us now.
+// 1242x375 pair, 118 us now.
 __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long* key, int W, int H, int* changed,
                                              int pass, int x0, int y0, VoronoiEdges& E)
 {
     const int lane = threadIdx.x, w = threadIdx.y;
     const int x = x0 + lane, yb = y0 + kBand * w;
-    const bool xin = x < W;
     auto load_key = [&](int px, int py) {
-        if (px < 0 || px >= W || py < 0 || py >= H) return kFar;
+        if (px < 0 || px >= W || py < 0 || py >= H) return 0ull;
         // halo keys belong to other tiles, which may lower them concurrently; any
         // value read is a valid upper bound
-        return min(*reinterpret_cast<const volatile unsigned long long*>(key + (size_t)py * W + px), kFar);
+        const unsigned long long v = *reinterpret_cast<const volatile unsigned long long*>(key + (size_t)py * W + px);
+        return v == kNone ? kFar : ((v >> kIdxBits) << 32) | (v & kIdxMask);
     };
     auto load_cost = [&](int px, int py) {
         return px >= 0 && px < W && py >= 0 && py < H ? (unsigned)cost[(size_t)py * W + px] : kWall;
     };
-    auto edge = [](unsigned a, unsigned b) { return a == kWall || b == kWall ? kWall : a + b; };
+    // weight of the step into a pixel of cost a from one of cost b
+    auto edge = [](unsigned a, unsigned b) { return a == kWall ? 0u : b == kWall ? kWall : a + b; };
     unsigned long long k[kBand], orig[kBand], side[kBand];  // side: the halo beside lanes 0 and 31
-    unsigned wl[kBand], wr[kBand], wv[kBand + 1];
+    unsigned wl[kBand], wr[kBand], wu[kBand], wd[kBand];  // weights of the steps into the lane's pixels
     {
         unsigned c[kBand + 2];
         const int xs = lane == 0 ? x - 1 : x + 1;  // used by lanes 0 and 31
@@ -172,9 +179,9 @@ __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long
             if (lane == 31) cr = cs;
             wl[r] = edge(c[r + 1], cl);
             wr[r] = edge(c[r + 1], cr);
+            wu[r] = edge(c[r + 1], c[r]);
+            wd[r] = edge(c[r + 1], c[r + 2]);
         }
-#pragma unroll
-        for (int r = 0; r <= kBand; ++r) wv[r] = edge(c[r], c[r + 1]);
     }
     // the halo rows above and below the tile, or the neighbouring bands' border rows
     const bool first = w == 0, last = w == kTile / kBand - 1;
@@ -195,12 +202,12 @@ __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long
             relax(b[r], l, wl[r]);
             relax(b[r], t, wr[r]);
         }
-        relax(b[0], up, wv[0]);
+        relax(b[0], up, wu[0]);
 #pragma unroll
-        for (int r = 1; r < kBand; ++r) relax(b[r], b[r - 1], wv[r]);
-        relax(b[kBand - 1], dn, wv[kBand]);
+        for (int r = 1; r < kBand; ++r) relax(b[r], b[r - 1], wu[r]);
+        relax(b[kBand - 1], dn, wd[kBand - 1]);
 #pragma unroll
-        for (int r = kBand - 2; r >= 0; --r) relax(b[r], b[r + 1], wv[r + 1]);
+        for (int r = kBand - 2; r >= 0; --r) relax(b[r], b[r + 1], wd[r]);
 #pragma unroll
         for (int r = 0; r < kBand; ++r) {
             ch |= b[r] < k[r];
@@ -223,8 +230,8 @@ __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long
     bool improved = false;
 #pragma unroll
     for (int r = 0; r < kBand; ++r)
-        if (k[r] < min(orig[r], kReal) && xin && yb + r < H) {
-            key[(size_t)(yb + r) * W + x] = k[r];
+        if (k[r] < orig[r]) {  // (never outside the frame: 0 there)
+            key[(size_t)(yb + r) * W + x] = ((k[r] >> 32) << kIdxBits) | (k[r] & kIdxMask);
             improved = true;
         }
     // (also keeps the next tile's border rows behind this tile's last sweep)
