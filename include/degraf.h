@@ -60,7 +60,8 @@ const char* dgf_strerror(int code);
 int dgf_version(void);
 
 /* device-side failures (dgf_device_status bits) */
-#define DGF_DEV_STAGE_WAIT 1u     /* a detection or pyramid block gave up waiting for its staging copies */
+#define DGF_DEV_STAGE_WAIT 1u     /* a detection or pyramid block gave up waiting for its staging copies, or a
+                                     block of the global-motion fit for the others */
 #define DGF_DEV_EPIC_PASSES 2u    /* epic_interpolate: the labelling did not settle (pass limit or barrier) */
 #define DGF_DEV_EPIC_CAPACITY 4u  /* epic_interpolate: a neighbourhood search outgrew its largest layout */
 

@@ -3,19 +3,27 @@
 // model used is a global affine motion fitted robustly to a sparse first pass and
 // used as every point's initial flow in the main pass.
 //
-// The fit is an IRLS loop of a few iterations, one launch each: 64 CTAs sum the
-// weighted normal equations of their points in FP64 (GB300's FP64 pipe is narrow,
+// The fit is an IRLS loop of a few iterations in one cooperative launch: 64 CTAs sum
+// the weighted normal equations of their points in FP64 (GB300's FP64 pipe is narrow,
 // so the sums are spread over the SMs) into per-CTA partials; the CTA that finishes
 // last (a ticket counter) adds the partials in CTA order, one thread per sum
-// (deterministic), and solves the two 3 x 3 systems. The state (affine, fitted flag,
-// go-on flag, ticket) lives in the workspace, so no host round trip separates the
-// stages: the main pass reads the fitted parameters from device memory.
+// (deterministic), solves the two 3 x 3 systems and releases the others, which wait
+// for it. The state (affine, fitted flag, go-on flag, ticket, released iteration) lives
+// in the workspace, so no host round trip separates the stages: the main pass reads
+// the fitted parameters from device memory.
+//
+// An iteration is a chain of FP64 latencies: sums, reduction, 64 additions, a solve of
+// some dozen dependent divisions and square roots. With a launch an iteration, xor
+// butterflies over all 13 sums and the two systems solved one after the other, the fit
+// of 12,669 points took 8 x 23.3 us and the gaps between launches; in one launch, with
+// halving exchanges and the systems solved in two lanes, 119 us. Same bits.
 #include "common.cuh"
 #include "batch.cuh"
 
 namespace {
 
 constexpr int kPartThreads = 256, kPartBlocks = 64;
+constexpr unsigned kWaitTries = 1u << 24;  // polls (20 ns naps) before a CTA stops waiting for the last one
 constexpr int kSums = 12;  // xx xy x yy y w | x qx, y qx, qx | x qy, y qy, qy
 
 // Cholesky solve of the 3 x 3 normal equations (row-major m[9]); a pivot below
@@ -48,7 +56,8 @@ __device__ bool solve3(const double* m, const double* b, double* x)
 }
 
 // State at the start of the workspace: a[6] (doubles), then int flags at byte 48
-// (1 = fitted) and byte 52 (1 = iterating), and the CTAs' ticket counter at byte 56.
+// (1 = fitted) and byte 52 (1 = iterating), the CTAs' ticket counter at byte 56 and the
+// number of finished iterations at byte 60.
 __global__ void gm_init_kernel(double* state)
 {
     state[0] = 1; state[1] = 0; state[2] = 0;
@@ -56,97 +65,137 @@ __global__ void gm_init_kernel(double* state)
     reinterpret_cast<int*>(state + 6)[0] = 0;
     reinterpret_cast<int*>(state + 6)[1] = 1;
     reinterpret_cast<unsigned*>(state + 7)[0] = 0;
+    reinterpret_cast<unsigned*>(state + 7)[1] = 0;
 }
 
-// IRLS iteration k: per-CTA sums over the points of the CTA's grid stride (point i
-// at pts[i * stride]); partial[blockIdx.x][0..11] = the 12 sums, [12] = the number of
-// weighted points. The last CTA to finish adds the partials in CTA order and solves
-// the two 3 x 3 systems; a step with fewer than 3 weighted points or a singular
-// matrix keeps the previous estimate and stops the loop.
-__global__ void __launch_bounds__(kPartThreads) gm_iteration_kernel(const float* pts, int stride, const float* flow,
-                                                                    const uint8_t* status, int n, int k, double c0,
-                                                                    double c_min, double* state, double* partial)
+// Sums of kSums + 1 values over the warp by halving exchanges: lanes 16 apart swap the
+// halves of their values and add, then lanes 8 apart quarters, and so on; a lane ends
+// with the total of value `lane / 2` (13 values padded to 16). Each total adds the lanes
+// in the order of an xor butterfly, with 16 additions a lane instead of 65.
+__device__ __forceinline__ double warp_totals(const double (&s)[kSums + 1])
+{
+    const int lane = threadIdx.x & 31;
+    double v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = j <= kSums ? s[j] : 0.0;
+#pragma unroll
+    for (int o = 16, n = 8; o >= 2; o >>= 1, n >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int j = 0; j < n; ++j) {
+            const double keep = hi ? v[n + j] : v[j], give = hi ? v[j] : v[n + j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// The IRLS iterations 0 .. iters - 1. Iteration k: per-CTA sums over the points of the
+// CTA's grid stride (point i at pts[i * stride]); partial[blockIdx.x][0..11] = the 12
+// sums, [12] = the number of weighted points. The last CTA to finish adds the partials in
+// CTA order and solves the two 3 x 3 systems; a step with fewer than 3 weighted points
+// or a singular matrix keeps the previous estimate and stops the loop. The waits are
+// bounded: a CTA that gives up sets DGF_DEV_STAGE_WAIT and leaves (the others follow).
+__global__ void __launch_bounds__(kPartThreads) gm_fit_kernel(const float* pts, int stride, const float* flow,
+                                                              const uint8_t* status, int n, int iters, double c0,
+                                                              double c_min, double* state, double* partial,
+                                                              unsigned* dev_status)
 {
     __shared__ double part[kPartThreads / 32][kSums + 1];
     __shared__ double tot[kSums + 1];
-    __shared__ int last;
+    __shared__ int last, go_on;
     int* flags = reinterpret_cast<int*>(state + 6);
     unsigned* ticket = reinterpret_cast<unsigned*>(state + 7);
-    if (!flags[1]) return;  // uniform: the fit has stopped
+    unsigned* done = ticket + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double a[6];
+    for (int k = 0; k < iters; ++k) {
+        double a[6];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) a[j] = state[j];
-    const double ck = fmax(c_min, ldexp(c0, -(k - 1)));
-    double s[kSums + 1];
+        for (int j = 0; j < 6; ++j) a[j] = __ldcg(state + j);
+        const double ck = fmax(c_min, ldexp(c0, -(k - 1)));
+        double s[kSums + 1];
 #pragma unroll
-    for (int j = 0; j <= kSums; ++j) s[j] = 0.0;
-    for (int i = blockIdx.x * kPartThreads + threadIdx.x; i < n; i += kPartBlocks * kPartThreads) {
-        if (status[i] != DGF_TRACKED) continue;
-        const float2 p = reinterpret_cast<const float2*>(pts)[(long long)i * stride];
-        const float2 f = reinterpret_cast<const float2*>(flow)[i];
-        const double x = p.x, y = p.y, qx = x + (double)f.x, qy = y + (double)f.y;
-        double w = 1.0;
-        if (k > 0) {
-            const double ex = a[0] * x + a[1] * y + a[2] - qx, ey = a[3] * x + a[4] * y + a[5] - qy;
-            const double e = sqrt(ex * ex + ey * ey);
-            if (e >= ck) continue;
-            const double u = 1.0 - (e / ck) * (e / ck);
-            w = u * u;
+        for (int j = 0; j <= kSums; ++j) s[j] = 0.0;
+        for (int i = blockIdx.x * kPartThreads + threadIdx.x; i < n; i += kPartBlocks * kPartThreads) {
+            if (status[i] != DGF_TRACKED) continue;
+            const float2 p = reinterpret_cast<const float2*>(pts)[(long long)i * stride];
+            const float2 f = reinterpret_cast<const float2*>(flow)[i];
+            const double x = p.x, y = p.y, qx = x + (double)f.x, qy = y + (double)f.y;
+            double w = 1.0;
+            if (k > 0) {
+                const double ex = a[0] * x + a[1] * y + a[2] - qx, ey = a[3] * x + a[4] * y + a[5] - qy;
+                const double e = sqrt(ex * ex + ey * ey);
+                if (e >= ck) continue;
+                const double u = 1.0 - (e / ck) * (e / ck);
+                w = u * u;
+            }
+            s[0] += w * x * x;
+            s[1] += w * x * y;
+            s[2] += w * x;
+            s[3] += w * y * y;
+            s[4] += w * y;
+            s[5] += w;
+            s[6] += w * x * qx;
+            s[7] += w * y * qx;
+            s[8] += w * qx;
+            s[9] += w * x * qy;
+            s[10] += w * y * qy;
+            s[11] += w * qy;
+            s[12] += 1.0;
         }
-        s[0] += w * x * x;
-        s[1] += w * x * y;
-        s[2] += w * x;
-        s[3] += w * y * y;
-        s[4] += w * y;
-        s[5] += w;
-        s[6] += w * x * qx;
-        s[7] += w * y * qx;
-        s[8] += w * qx;
-        s[9] += w * x * qy;
-        s[10] += w * y * qy;
-        s[11] += w * qy;
-        s[12] += 1.0;
+        // fixed-order reduction: over each warp, then one thread a sum over the warps
+        const double t = warp_totals(s);
+        if (!(lane & 1) && lane / 2 <= kSums) part[warp][lane / 2] = t;
+        __syncthreads();
+        if (threadIdx.x <= kSums) {
+            double t = 0.0;
+            for (int w = 0; w < kPartThreads / 32; ++w) t += part[w][threadIdx.x];
+            partial[blockIdx.x * (kSums + 1) + threadIdx.x] = t;
+            __threadfence();  // the partial is visible device-wide before this CTA's ticket
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == (unsigned)(k + 1) * gridDim.x - 1;
+        __syncthreads();
+        if (last) {
+            // every other CTA's partial was written before its ticket
+            __threadfence();
+            if (threadIdx.x <= kSums) {
+                double t = 0.0;
+#pragma unroll 16
+                for (int b = 0; b < kPartBlocks; ++b) t += __ldcg(partial + b * (kSums + 1) + threadIdx.x);
+                tot[threadIdx.x] = t;
+            }
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                // lanes 0 and 1 solve for the two rows of the affine at once
+                const double m[9] = {tot[0], tot[1], tot[2], tot[1], tot[3], tot[4], tot[2], tot[4], tot[5]};
+                const int r = lane & 1;
+                const double rhs[3] = {tot[6 + 3 * r], tot[7 + 3 * r], tot[8 + 3 * r]};
+                double x[3];
+                const bool ok = __all_sync(0xffffffffu, !(tot[12] < 3.0) && solve3(m, rhs, x));
+                if (ok && lane < 2) {
+                    for (int j = 0; j < 3; ++j) state[3 * r + j] = x[j];
+                    flags[0] = 1;
+                }
+                if (!ok && lane == 0) flags[1] = 0;  // keep the previous estimate
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) atomicExch(done, (unsigned)(k + 1));
+            }
+        }
+        if (threadIdx.x == 0) {
+            int ok = 0;
+            for (unsigned i = 0; i < kWaitTries && !ok; ++i) {
+                ok = *reinterpret_cast<volatile unsigned*>(done) >= (unsigned)(k + 1);
+                if (!ok) __nanosleep(20);
+            }
+            __threadfence();
+            if (!ok && dev_status) atomicOr(dev_status, (unsigned)DGF_DEV_STAGE_WAIT);
+            go_on = ok && *reinterpret_cast<volatile int*>(flags + 1);
+        }
+        __syncthreads();
+        if (!go_on) return;  // uniform: the fit has stopped
     }
-    // fixed-order reduction: xor butterfly in each warp, then one thread a sum over the warps
-#pragma unroll
-    for (int j = 0; j <= kSums; ++j)
-        for (int o = 16; o > 0; o >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
-    if (lane == 0)
-#pragma unroll
-        for (int j = 0; j <= kSums; ++j) part[warp][j] = s[j];
-    __syncthreads();
-    if (threadIdx.x <= kSums) {
-        double t = 0.0;
-        for (int w = 0; w < kPartThreads / 32; ++w) t += part[w][threadIdx.x];
-        partial[blockIdx.x * (kSums + 1) + threadIdx.x] = t;
-        __threadfence();  // the partial is visible device-wide before this CTA's ticket
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    // the last CTA: every other CTA's partial was written before its ticket
-    __threadfence();
-    if (threadIdx.x <= kSums) {
-        double t = 0.0;
-#pragma unroll 8
-        for (int b = 0; b < kPartBlocks; ++b) t += __ldcg(partial + b * (kSums + 1) + threadIdx.x);
-        tot[threadIdx.x] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    *ticket = 0;  // for the next iteration's launch
-    const double m[9] = {tot[0], tot[1], tot[2], tot[1], tot[3], tot[4], tot[2], tot[4], tot[5]};
-    const double bx[3] = {tot[6], tot[7], tot[8]}, by[3] = {tot[9], tot[10], tot[11]};
-    double sx[3], sy[3];
-    if (tot[12] < 3.0 || !solve3(m, bx, sx) || !solve3(m, by, sy)) {
-        flags[1] = 0;  // keep the previous estimate
-        return;
-    }
-    state[0] = sx[0]; state[1] = sx[1]; state[2] = sx[2];
-    state[3] = sy[0]; state[4] = sy[1]; state[5] = sy[2];
-    flags[0] = 1;
 }
 
 bool gm_params_ok(const dgf_gm_params* g)
@@ -218,10 +267,16 @@ extern "C" int rlof_track_gm(const void* pyr1, const void* pyr2, int W, int H, i
     if ((rc = dgf::launch_track(first, &deep, stream)) != DGF_OK) return rc;
     // 2. robust affine fit
     double* partial = reinterpret_cast<double*>(ws + partial_offset(n_sub));
+    unsigned* dev_status = dgf::status_word();  // (null: the kernel records nothing)
     gm_init_kernel<<<1, 1, 0, stream>>>(affine);
-    for (int k = 0; k < g->iters; ++k) {
-        gm_iteration_kernel<<<kPartBlocks, kPartThreads, 0, stream>>>(pts, g->stride, sub_flow, sub_status,
-                                                                       (int)n_sub, k, g->c0, g->c_min, affine, partial);
+    {
+        int n_pts = (int)n_sub, stride = g->stride, iters = g->iters;
+        double c0 = g->c0, c_min = g->c_min;
+        void* args[] = {(void*)&pts, (void*)&stride, (void*)&sub_flow, (void*)&sub_status, (void*)&n_pts, (void*)&iters,
+                        (void*)&c0, (void*)&c_min, (void*)&affine, (void*)&partial, (void*)&dev_status};
+        if (cudaLaunchCooperativeKernel((const void*)gm_fit_kernel, dim3(kPartBlocks), dim3(kPartThreads), args, 0,
+                                        stream) != cudaSuccess)
+            return DGF_ERR_CUDA;
     }
     if ((rc = dgf::launch_status()) != DGF_OK) return rc;
     // 3. main pass from the prior
