@@ -57,7 +57,7 @@ constexpr unsigned kNoLink = 0xffffffffu;  // min link weight of a seed without 
 
 // Device status bits (any of them makes the call return DGF_ERR_DEVICE).
 enum : int { kErrFrontier = 1, kErrFill = 4, kErrRange = 8, kErrPasses = 16, kErrSync = 32 };
-constexpr unsigned kBarrierTries = 1u << 24;  // polls (100 ns naps) before a grid barrier gives up
+constexpr unsigned kBarrierTries = 1u << 24;  // polls (20 ns naps) before a grid barrier gives up
 
 __device__ __forceinline__ bool is_tracked(uint8_t s) { return s == DGF_TRACKED || s == DGF_MAXITER; }
 
@@ -135,14 +135,20 @@ struct VoronoiEdges {
 // every third sweep is closed by a barrier before and a vote after it: once it changes
 // nothing, every pixel was checked against final neighbours. Improved keys are
 // written back (the tile's pixels are written by nobody else); counts the tile in
-// changed[pass] if any key improved. Called by every thread of the block.
+// changed[pass] if any key improved. Called by every thread of the block. With fresh
+// unset, T still holds the tile's keys and weights from the block's last pass (a block
+// that owns one tile loads them once and then only the halo).
 // What bounds it is the latency of one sweep times the longest path inside a tile
 // (shortest paths through seedless areas wind for 50 pixels and more). With a thread
 // per four scattered pixels, all keys in shared memory and two barriers a sweep, a
 // sweep took about 1,250 cycles and moved a path one pixel: 227 us of labelling on the
-// 1242x375 pair, 118 us now.
+// 1242x375 pair, about 110 us now.
+struct VoronoiBand {
+    unsigned long long k[kBand];
+    unsigned wl[kBand], wr[kBand], wu[kBand], wd[kBand];  // weights of the steps into the lane's pixels
+};
 __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long* key, int W, int H, int* changed,
-                                             int pass, int x0, int y0, VoronoiEdges& E)
+                                             int pass, int x0, int y0, VoronoiEdges& E, VoronoiBand& T, bool fresh)
 {
     const int lane = threadIdx.x, w = threadIdx.y;
     const int x = x0 + lane, yb = y0 + kBand * w;
@@ -158,17 +164,13 @@ __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long
     };
     // weight of the step into a pixel of cost a from one of cost b
     auto edge = [](unsigned a, unsigned b) { return a == kWall ? 0u : b == kWall ? kWall : a + b; };
-    unsigned long long k[kBand], orig[kBand], side[kBand];  // side: the halo beside lanes 0 and 31
-    unsigned wl[kBand], wr[kBand], wu[kBand], wd[kBand];  // weights of the steps into the lane's pixels
-    {
+    unsigned long long(&k)[kBand] = T.k;
+    const int xs = lane == 0 ? x - 1 : x + 1;  // beside the tile, for lanes 0 and 31
+    const bool outer = lane == 0 || lane == 31;
+    if (fresh) {
         unsigned c[kBand + 2];
-        const int xs = lane == 0 ? x - 1 : x + 1;  // used by lanes 0 and 31
-        const bool outer = lane == 0 || lane == 31;
 #pragma unroll
-        for (int r = 0; r < kBand; ++r) {
-            orig[r] = k[r] = load_key(x, yb + r);
-            side[r] = outer ? load_key(xs, yb + r) : kFar;
-        }
+        for (int r = 0; r < kBand; ++r) k[r] = load_key(x, yb + r);
 #pragma unroll
         for (int r = 0; r < kBand + 2; ++r) c[r] = load_cost(x, yb + r - 1);
 #pragma unroll
@@ -177,11 +179,17 @@ __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long
             unsigned cl = __shfl_up_sync(0xffffffffu, c[r + 1], 1), cr = __shfl_down_sync(0xffffffffu, c[r + 1], 1);
             if (lane == 0) cl = cs;
             if (lane == 31) cr = cs;
-            wl[r] = edge(c[r + 1], cl);
-            wr[r] = edge(c[r + 1], cr);
-            wu[r] = edge(c[r + 1], c[r]);
-            wd[r] = edge(c[r + 1], c[r + 2]);
+            T.wl[r] = edge(c[r + 1], cl);
+            T.wr[r] = edge(c[r + 1], cr);
+            T.wu[r] = edge(c[r + 1], c[r]);
+            T.wd[r] = edge(c[r + 1], c[r + 2]);
         }
+    }
+    unsigned long long orig[kBand], side[kBand];  // side: the halo beside lanes 0 and 31
+#pragma unroll
+    for (int r = 0; r < kBand; ++r) {
+        orig[r] = k[r];
+        side[r] = outer ? load_key(xs, yb + r) : kFar;
     }
     // the halo rows above and below the tile, or the neighbouring bands' border rows
     const bool first = w == 0, last = w == kTile / kBand - 1;
@@ -199,15 +207,15 @@ __device__ __forceinline__ void voronoi_tile(const int* cost, unsigned long long
             if (lane == 0) l = side[r];
             if (lane == 31) t = side[r];
             b[r] = k[r];
-            relax(b[r], l, wl[r]);
-            relax(b[r], t, wr[r]);
+            relax(b[r], l, T.wl[r]);
+            relax(b[r], t, T.wr[r]);
         }
-        relax(b[0], up, wu[0]);
+        relax(b[0], up, T.wu[0]);
 #pragma unroll
-        for (int r = 1; r < kBand; ++r) relax(b[r], b[r - 1], wu[r]);
-        relax(b[kBand - 1], dn, wd[kBand - 1]);
+        for (int r = 1; r < kBand; ++r) relax(b[r], b[r - 1], T.wu[r]);
+        relax(b[kBand - 1], dn, T.wd[kBand - 1]);
 #pragma unroll
-        for (int r = kBand - 2; r >= 0; --r) relax(b[r], b[r + 1], wd[r]);
+        for (int r = kBand - 2; r >= 0; --r) relax(b[r], b[r + 1], T.wd[r]);
 #pragma unroll
         for (int r = 0; r < kBand; ++r) {
             ch |= b[r] < k[r];
@@ -254,7 +262,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target)
                 ok = 1;
                 break;
             }
-            __nanosleep(100);
+            __nanosleep(20);
         }
         __threadfence();
         s_ok = ok;
@@ -272,11 +280,13 @@ __global__ void __launch_bounds__(kThreads, 4) epic_voronoi_kernel(const int* co
                                                                 int* changed, unsigned* sync_count, int* err)
 {
     __shared__ VoronoiEdges edges;
+    VoronoiBand band;
     const int tiles_x = (W + kTile - 1) / kTile, n_tiles = tiles_x * ((H + kTile - 1) / kTile);
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0;
     for (int pass = 0; pass < kMaxPasses; ++pass) {
         for (int t = blockIdx.x; t < n_tiles; t += gridDim.x)
-            voronoi_tile(cost, key, W, H, changed, pass, (t % tiles_x) * kTile, (t / tiles_x) * kTile, edges);
+            voronoi_tile(cost, key, W, H, changed, pass, (t % tiles_x) * kTile, (t / tiles_x) * kTile, edges, band,
+                         pass == 0 || n_tiles > (int)gridDim.x);
         if (!grid_barrier(sync_count, (unsigned)(pass + 1) * gridDim.x)) {
             if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(err, kErrSync);
             return;
