@@ -66,6 +66,7 @@ struct TrackJob {
 struct TrackBatch {
     int levels, pyr_levels, radius, max_iter, es;  // pyr_levels: levels the pyramids were built with
     float eps2, ha, hc, inv_cb, min_eig, cross_tau;  // cross_tau > 0: adaptive cross-based support
+    float r_in;         // residuals of at most r_in in magnitude have Hampel weight exactly 1
     int n_jobs, total;  // jobs, and points over all jobs
     TrackJob jobs[kMaxBatchPairs];
 };
