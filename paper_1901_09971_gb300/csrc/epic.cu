@@ -10,17 +10,16 @@
 //   2. seeds claim their pixels (atomicMin on (distance 0, index)), then keep a
 //      pixel only where they hold it;
 //   3. geodesic Voronoi labelling by tile-local relaxation: 32 x 32 tiles iterate
-//      min-plus updates of the packed key (distance << 24 | seed) in shared memory
-//      until they are locally stable, write improvements back with atomicMin and
-//      count them; passes repeat until one changes nothing (the host reads the
-//      counter every four passes). Relaxation converges to the unique fixed
-//      point, the lexicographic (distance, seed) minimum, whatever the order;
+//      min-plus updates of the (distance, seed) keys in registers until they are
+//      locally stable, write improvements back and count them; one cooperative launch
+//      repeats passes until one changes nothing. Relaxation converges to the unique
+//      fixed point, the lexicographic (distance, seed) minimum, whatever the order;
 //   4-6. seed graph: links of 4-adjacent pixels in different cells are counted,
 //      scanned into offsets (three launches: block scans, a scan of the block
 //      totals, the block offsets added) and filled into per-seed lists;
-//   7-8. each list keeps one link per neighbour (its smallest weight), and every
-//      link records where its neighbour's list lies, so a search reads a popped
-//      seed's links without first loading its list bounds;
+//   7-8. each list keeps one link per neighbour (its smallest weight), in a 16-byte
+//      record with the neighbour's own smallest weight, so a search discovers a seed
+//      with one load;
 //   9. per seed, one warp runs Dijkstra over the seed graph with batch settling
 //      (every frontier seed within its smallest incoming link of the frontier
 //      minimum is final, so about 14 steps settle the 128 nearest instead of 128
