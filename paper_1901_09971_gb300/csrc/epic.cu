@@ -76,6 +76,7 @@ __device__ __forceinline__ void begin_after()
 
 // Launches a kernel that calls begin_after first. Not for kernels that read what the call
 // writes by __ldg (the search): its data must not change while the kernel is resident.
+// With plain loads the search gains nothing from it (107 and 815 us).
 template <typename... P, typename... A>
 void launch_next(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t stream, A... args)
 {

@@ -5,6 +5,7 @@ end. Indices and distances are exact integers; models within 1e-9 and the dense 
 within 1e-4 px, as for every EPIC case."""
 import numpy as np
 import pytest
+import torch
 
 from test_gpu_epic import assert_parity, dgf, run_both  # noqa: F401
 from test_oracle_epic import random_matches, textured
@@ -57,3 +58,43 @@ def test_weights_past_the_table(dgf):  # noqa: F811
     g, o = run_both(dgf, img, pts, flow, status, k=40, cost_base=4096, cost_gain=2, a=0.05)
     assert np.median(g["knn_dist"][g["knn_dist"] > 0]) > 16384
     assert_parity(g, o)
+
+
+def test_calls_in_sequence_share_a_workspace(dgf):  # noqa: F811
+    """Launches of a call overlap with the kernels before them: calls of other sizes in a
+    row on one dirty workspace, and the same in a captured graph, give the bits of calls
+    alone on zeroed ones."""
+    prm = dgf.EpicParams(k=24)
+    sets = []
+    for W, H, n in ((256, 128, 1900), (40, 33, 60), (203, 97, 3000), (64, 64, 500)):
+        pts, flow, status = random_matches(W, H, n, n)
+        sets.append([torch.from_numpy(v).cuda() for v in (textured(W, H, n), pts.astype(np.float32),
+                                                          flow.astype(np.float32), status)])
+    room = max(dgf.epic_workspace_bytes(s[0].shape[1], s[0].shape[0], len(s[1])) for s in sets)
+    alone = []
+    for s in sets:
+        alone.append(dgf.epic_interpolate(*s, prm, workspace=torch.zeros(room, dtype=torch.uint8, device="cuda")))
+        torch.cuda.synchronize()
+    ws = torch.full((room,), 0xAB, dtype=torch.uint8, device="cuda")
+    outs = [torch.full_like(d, -7.0) for d in alone + alone]
+
+    def run():
+        for i, o in enumerate(outs):
+            dgf.epic_interpolate(*sets[i % len(sets)], prm, workspace=ws, out=o)
+
+    def check():
+        torch.cuda.synchronize()
+        for i, o in enumerate(outs):
+            assert torch.equal(o, alone[i % len(sets)])
+            o.fill_(-7.0)
+
+    run()
+    check()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    graph.replay()
+    check()
+    graph.replay()
+    check()
+    assert dgf.device_status() == 0
