@@ -34,6 +34,7 @@
 
 #include "common.cuh"
 #include "batch.cuh"
+#include "track_index.cuh"
 
 namespace rlof_detail {
 
@@ -78,9 +79,9 @@ __device__ __forceinline__ float group_sum(float v, unsigned mask)
 }
 
 // Per-warp scratch of the group reduction: one row of 16 partial sums per lane and
-// 16 totals per group; and the groups' kept factors. Rows are 20 floats apart, so the 16-byte accesses of eight
-// consecutive lanes start in distinct quads of banks.
-constexpr int kRowStride = 20;
+// 16 totals per group; and the groups' kept factors. Rows are 20 floats apart, so the
+// 16-byte accesses of eight consecutive lanes start in distinct quads of banks.
+using dgf::kRowStride;
 struct alignas(16) WarpScratch {
     float rows[32 * kRowStride];
     float totals[4 * 16];
@@ -101,7 +102,8 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b)
 // group; the G / 4 lanes holding the same block combine their partial sums with
 // xor shuffles; lanes 0..3 publish the four block totals, which every lane of the
 // group then reads back, so all lanes receive the same bits. Groups of a warp use
-// disjoint rows and totals, so diverged groups never meet at a barrier.
+// disjoint rows and totals, here and in group_allreduce4, so diverged groups never
+// meet at a barrier, and a group may reduce 4 values while another reduces 16.
 template <int G>
 __device__ __forceinline__ void group_allreduce16(const float (&v)[16], float (&h)[16], unsigned mask, int lane,
                                                   WarpScratch& ws)
@@ -145,17 +147,16 @@ __device__ __forceinline__ void group_allreduce16(const float (&v)[16], float (&
 // The same for 4 values (h[k] = total of v[k]), added in the same order as
 // group_allreduce16 adds a block: lane l takes value l & 3 of the rows
 // 4 (l >> 2) .. +3, the lanes holding the same value combine with xor shuffles, and
-// lanes 0..3 hand the totals round. A value's lanes lie side by side, values 40 floats
-// apart (conflict-free 4-byte stores and 16-byte reads).
+// lanes 0..3 hand the totals round. The values lie inside the group's rows (short_place).
 template <int G>
 __device__ __forceinline__ void group_allreduce4(const float (&v)[4], float (&h)[4], unsigned mask, int lane,
                                                  WarpScratch& ws)
 {
     const int wl = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) ws.rows[40 * i + wl] = v[i];
+    for (int i = 0; i < 4; ++i) ws.rows[dgf::short_place(wl, lane, i)] = v[i];
     __syncwarp(mask);
-    const float4 r = *reinterpret_cast<const float4*>(ws.rows + 40 * (wl & 3) + (wl & ~3));
+    const float4 r = *reinterpret_cast<const float4*>(ws.rows + dgf::short_read(wl, lane));
     float s = __fadd_rn(__fadd_rn(__fadd_rn(r.x, r.y), r.z), r.w);
 #pragma unroll
     for (int o = 4; o < G; o <<= 1) s = __fadd_rn(s, __shfl_xor_sync(mask, s, o));
