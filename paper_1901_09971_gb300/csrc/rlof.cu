@@ -995,13 +995,14 @@ __device__ __forceinline__ bool setup_level(Support<SLP>& S, const LevelView<TS>
     constexpr int FG = first_generic_slot<G, SLP, RC>();
     const int side = 2 * R + 1;
     const float fx0 = floorf(plx), fy0 = floorf(ply);
-    const int bx = (int)fx0 - R, by = (int)fy0 - R;
+    static_assert(dgf::kFar > 2 * DGF_MAX_RADIUS + 3 + dgf::kApron, "far points are outside the border");
+    const int bx = dgf::tap_origin(fx0, R, L.W), by = dgf::tap_origin(fy0, R, L.H);
     const PairWeights pw(plx - fx0, ply - fy0);
     // the template's taps read without clamping when they lie within the planes'
     // replicated border, as they do for every point inside the frame (points given
     // outside it take the clamped reads)
-    const bool direct = bx >= -dgf::kApron && bx + 2 * R + 2 <= L.W + dgf::kApron - 1 && by >= -dgf::kApron &&
-                        by + 2 * R + 1 <= L.H + dgf::kApron - 1;
+    const bool direct = dgf::taps_inside(bx, 2 * R + 3, L.W, dgf::kApron) &&
+                        dgf::taps_inside(by, 2 * R + 2, L.H, dgf::kApron);
     float2 g00 = f2(0.f), g01 = f2(0.f), g11 = f2(0.f);
     float kept = 0.f;  // cross-based support: kept samples of the lane
     if constexpr (RunLayout<G, RC>::on && MODEL == 4 && sizeof(TS) == 4 && !CROSS) {
