@@ -133,6 +133,21 @@ inline int launch_status() {
     return e == cudaSuccess ? DGF_OK : DGF_ERR_CUDA;
 }
 
+// Blocks for a cooperative launch of a kernel without dynamic shared memory: `wanted`, or
+// as many as the device (or the share of it that the process may use) holds at once if
+// that is less; 0 when it cannot be found out.
+template <typename K>
+inline unsigned cooperative_blocks(K kernel, int threads, long long wanted)
+{
+    int per_sm = 0, dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess)
+        return 0;
+    const long long fit = (long long)per_sm * sms;
+    return (unsigned)(wanted < fit ? wanted : fit);
+}
+
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 }  // namespace dgf

@@ -1390,14 +1390,9 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
     // geodesic Voronoi labelling: passes until one changes nothing, in one
     // cooperative launch of as many blocks as can be resident (at most one a tile)
     {
-        int per_sm = 0, dev = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, epic_voronoi_kernel, kThreads, 0) != cudaSuccess ||
-            per_sm < 1)
-            return DGF_ERR_CUDA;
         const long long tiles = (long long)((W + kTile - 1) / kTile) * ((H + kTile - 1) / kTile);
-        const unsigned grid = (unsigned)std::min<long long>(tiles, (long long)per_sm * sms);
+        const unsigned grid = dgf::cooperative_blocks(epic_voronoi_kernel, kThreads, tiles);
+        if (grid < 1) return DGF_ERR_CUDA;
         const dim3 block(32, 8);
         void* args[] = {(void*)&cost, (void*)&key, (void*)&W, (void*)&H, (void*)&changed, (void*)&sync_count,
                         (void*)&err};

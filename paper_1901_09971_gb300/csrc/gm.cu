@@ -3,12 +3,14 @@
 // model used is a global affine motion fitted robustly to a sparse first pass and
 // used as every point's initial flow in the main pass.
 //
-// The fit is an IRLS loop of a few iterations in one cooperative launch: 64 CTAs sum
-// the weighted normal equations of their points in FP64 (GB300's FP64 pipe is narrow,
-// so the sums are spread over the SMs) into per-CTA partials; the CTA that finishes
-// last (a ticket counter) adds the partials in CTA order, one thread per sum
-// (deterministic), solves the two 3 x 3 systems and releases the others, which wait
-// for it. The state (affine, fitted flag, go-on flag, ticket, released iteration) lives
+// The fit is an IRLS loop of a few iterations in one cooperative launch: the points form
+// 64 parts, a CTA sums the weighted normal equations of one part in FP64 (GB300's FP64
+// pipe is narrow, so the sums are spread over the SMs; of several parts, one after the
+// other, where fewer than 64 CTAs are resident at once, as in a process that may use
+// only some of the SMs) into the part's partial; the CTA that finishes last (a ticket
+// counter) adds the partials in the parts' order, one thread per sum (deterministic, and
+// the same bits for any number of CTAs), solves the two 3 x 3 systems and releases the
+// others, which wait for it. The state (affine, fitted flag, go-on flag, ticket, released iteration) lives
 // in the workspace, so no host round trip separates the stages: the main pass reads
 // the fitted parameters from device memory.
 //
@@ -22,7 +24,7 @@
 
 namespace {
 
-constexpr int kPartThreads = 256, kPartBlocks = 64;
+constexpr int kPartThreads = 256, kParts = 64;
 constexpr unsigned kWaitTries = 1u << 24;  // polls (20 ns naps) before a CTA stops waiting for the last one
 constexpr int kSums = 12;  // xx xy x yy y w | x qx, y qx, qx | x qy, y qy, qy
 
@@ -90,10 +92,10 @@ __device__ __forceinline__ double warp_totals(const double (&s)[kSums + 1])
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// The IRLS iterations 0 .. iters - 1. Iteration k: per-CTA sums over the points of the
-// CTA's grid stride (point i at pts[i * stride]); partial[blockIdx.x][0..11] = the 12
-// sums, [12] = the number of weighted points. The last CTA to finish adds the partials in
-// CTA order and solves the two 3 x 3 systems; a step with fewer than 3 weighted points
+// The IRLS iterations 0 .. iters - 1. Iteration k: sums over the points of part b, every
+// kParts-th run of kPartThreads points (point i at pts[i * stride]); partial[b][0..11] =
+// the 12 sums, [12] = the number of weighted points. The last CTA to finish adds the
+// partials in the parts' order and solves the two 3 x 3 systems; a step with fewer than 3 weighted points
 // or a singular matrix keeps the previous estimate and stops the loop. The waits are
 // bounded: a CTA that gives up sets DGF_DEV_STAGE_WAIT and leaves (the others follow).
 __global__ void __launch_bounds__(kPartThreads) gm_fit_kernel(const float* pts, int stride, const float* flow,
@@ -113,46 +115,49 @@ __global__ void __launch_bounds__(kPartThreads) gm_fit_kernel(const float* pts, 
 #pragma unroll
         for (int j = 0; j < 6; ++j) a[j] = __ldcg(state + j);
         const double ck = fmax(c_min, ldexp(c0, -(k - 1)));
-        double s[kSums + 1];
+        for (int b = blockIdx.x; b < kParts; b += gridDim.x) {
+            double s[kSums + 1];
 #pragma unroll
-        for (int j = 0; j <= kSums; ++j) s[j] = 0.0;
-        for (int i = blockIdx.x * kPartThreads + threadIdx.x; i < n; i += kPartBlocks * kPartThreads) {
-            if (status[i] != DGF_TRACKED) continue;
-            const float2 p = reinterpret_cast<const float2*>(pts)[(long long)i * stride];
-            const float2 f = reinterpret_cast<const float2*>(flow)[i];
-            const double x = p.x, y = p.y, qx = x + (double)f.x, qy = y + (double)f.y;
-            double w = 1.0;
-            if (k > 0) {
-                const double ex = a[0] * x + a[1] * y + a[2] - qx, ey = a[3] * x + a[4] * y + a[5] - qy;
-                const double e = sqrt(ex * ex + ey * ey);
-                if (e >= ck) continue;
-                const double u = 1.0 - (e / ck) * (e / ck);
-                w = u * u;
+            for (int j = 0; j <= kSums; ++j) s[j] = 0.0;
+            for (int i = b * kPartThreads + threadIdx.x; i < n; i += kParts * kPartThreads) {
+                if (status[i] != DGF_TRACKED) continue;
+                const float2 p = reinterpret_cast<const float2*>(pts)[(long long)i * stride];
+                const float2 f = reinterpret_cast<const float2*>(flow)[i];
+                const double x = p.x, y = p.y, qx = x + (double)f.x, qy = y + (double)f.y;
+                double w = 1.0;
+                if (k > 0) {
+                    const double ex = a[0] * x + a[1] * y + a[2] - qx, ey = a[3] * x + a[4] * y + a[5] - qy;
+                    const double e = sqrt(ex * ex + ey * ey);
+                    if (e >= ck) continue;
+                    const double u = 1.0 - (e / ck) * (e / ck);
+                    w = u * u;
+                }
+                s[0] += w * x * x;
+                s[1] += w * x * y;
+                s[2] += w * x;
+                s[3] += w * y * y;
+                s[4] += w * y;
+                s[5] += w;
+                s[6] += w * x * qx;
+                s[7] += w * y * qx;
+                s[8] += w * qx;
+                s[9] += w * x * qy;
+                s[10] += w * y * qy;
+                s[11] += w * qy;
+                s[12] += 1.0;
             }
-            s[0] += w * x * x;
-            s[1] += w * x * y;
-            s[2] += w * x;
-            s[3] += w * y * y;
-            s[4] += w * y;
-            s[5] += w;
-            s[6] += w * x * qx;
-            s[7] += w * y * qx;
-            s[8] += w * qx;
-            s[9] += w * x * qy;
-            s[10] += w * y * qy;
-            s[11] += w * qy;
-            s[12] += 1.0;
+            // fixed-order reduction: over each warp, then one thread a sum over the warps
+            const double v = warp_totals(s);
+            __syncthreads();  // the part before has been read
+            if (!(lane & 1) && lane / 2 <= kSums) part[warp][lane / 2] = v;
+            __syncthreads();
+            if (threadIdx.x <= kSums) {
+                double t = 0.0;
+                for (int w = 0; w < kPartThreads / 32; ++w) t += part[w][threadIdx.x];
+                partial[b * (kSums + 1) + threadIdx.x] = t;
+            }
         }
-        // fixed-order reduction: over each warp, then one thread a sum over the warps
-        const double t = warp_totals(s);
-        if (!(lane & 1) && lane / 2 <= kSums) part[warp][lane / 2] = t;
-        __syncthreads();
-        if (threadIdx.x <= kSums) {
-            double t = 0.0;
-            for (int w = 0; w < kPartThreads / 32; ++w) t += part[w][threadIdx.x];
-            partial[blockIdx.x * (kSums + 1) + threadIdx.x] = t;
-            __threadfence();  // the partial is visible device-wide before this CTA's ticket
-        }
+        if (threadIdx.x <= kSums) __threadfence();  // the partials are visible device-wide before this CTA's ticket
         __syncthreads();
         if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == (unsigned)(k + 1) * gridDim.x - 1;
         __syncthreads();
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(kPartThreads) gm_fit_kernel(const float* pts, 
             if (threadIdx.x <= kSums) {
                 double t = 0.0;
 #pragma unroll 16
-                for (int b = 0; b < kPartBlocks; ++b) t += __ldcg(partial + b * (kSums + 1) + threadIdx.x);
+                for (int b = 0; b < kParts; ++b) t += __ldcg(partial + b * (kSums + 1) + threadIdx.x);
                 tot[threadIdx.x] = t;
             }
             __syncthreads();
@@ -205,11 +210,11 @@ bool gm_params_ok(const dgf_gm_params* g)
 }
 
 // Workspace layout: [a[6], flags, ticket; 256 B] [first-pass flow, n_sub x 8 B] [first-pass status, n_sub B]
-// [per-CTA partial sums, 64 x 13 doubles]
+// [the parts' partial sums, 64 x 13 doubles]
 size_t flow_offset() { return 256; }
 size_t status_offset(long long n_sub) { return dgf::round_up(flow_offset() + (size_t)n_sub * 8, 256); }
 size_t partial_offset(long long n_sub) { return dgf::round_up(status_offset(n_sub) + (size_t)n_sub, 256); }
-constexpr size_t kPartialBytes = (size_t)kPartBlocks * (kSums + 1) * 8;
+constexpr size_t kPartialBytes = (size_t)kParts * (kSums + 1) * 8;
 
 }  // namespace
 
@@ -274,8 +279,10 @@ extern "C" int rlof_track_gm(const void* pyr1, const void* pyr2, int W, int H, i
         double c0 = g->c0, c_min = g->c_min;
         void* args[] = {(void*)&pts, (void*)&stride, (void*)&sub_flow, (void*)&sub_status, (void*)&n_pts, (void*)&iters,
                         (void*)&c0, (void*)&c_min, (void*)&affine, (void*)&partial, (void*)&dev_status};
-        if (cudaLaunchCooperativeKernel((const void*)gm_fit_kernel, dim3(kPartBlocks), dim3(kPartThreads), args, 0,
-                                        stream) != cudaSuccess)
+        const unsigned grid = dgf::cooperative_blocks(gm_fit_kernel, kPartThreads, kParts);
+        if (grid < 1) return DGF_ERR_CUDA;
+        if (cudaLaunchCooperativeKernel((const void*)gm_fit_kernel, dim3(grid), dim3(kPartThreads), args, 0, stream) !=
+            cudaSuccess)
             return DGF_ERR_CUDA;
     }
     if ((rc = dgf::launch_status()) != DGF_OK) return rc;
