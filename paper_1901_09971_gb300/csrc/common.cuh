@@ -148,6 +148,18 @@ inline unsigned cooperative_blocks(K kernel, int threads, long long wanted)
     return (unsigned)(wanted < fit ? wanted : fit);
 }
 
+// Launches a kernel whose blocks wait for one another on `grid` blocks (0: the query above
+// failed). A refused launch leaves no error behind that a later call would report.
+inline int launch_cooperative(const void* kernel, unsigned grid, dim3 block, void** args, cudaStream_t stream)
+{
+    if (grid < 1) {
+        (void)cudaGetLastError();
+        return DGF_ERR_CUDA;
+    }
+    (void)cudaLaunchCooperativeKernel(kernel, dim3(grid), block, args, 0, stream);
+    return launch_status();
+}
+
 inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
 }  // namespace dgf

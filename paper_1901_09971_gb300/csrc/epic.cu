@@ -1392,13 +1392,10 @@ extern "C" int epic_interpolate(const uint8_t* img, int W, int H, int pitch, con
     {
         const long long tiles = (long long)((W + kTile - 1) / kTile) * ((H + kTile - 1) / kTile);
         const unsigned grid = dgf::cooperative_blocks(epic_voronoi_kernel, kThreads, tiles);
-        if (grid < 1) return DGF_ERR_CUDA;
         const dim3 block(32, 8);
         void* args[] = {(void*)&cost, (void*)&key, (void*)&W, (void*)&H, (void*)&changed, (void*)&sync_count,
                         (void*)&err};
-        if (cudaLaunchCooperativeKernel((const void*)epic_voronoi_kernel, dim3(grid), block, args, 0, stream) !=
-            cudaSuccess)
-            return DGF_ERR_CUDA;
+        if ((rc = dgf::launch_cooperative((const void*)epic_voronoi_kernel, grid, block, args, stream)) != DGF_OK) return rc;
     }
 
     if (n > 0) {

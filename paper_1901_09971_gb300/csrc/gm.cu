@@ -280,12 +280,9 @@ extern "C" int rlof_track_gm(const void* pyr1, const void* pyr2, int W, int H, i
         void* args[] = {(void*)&pts, (void*)&stride, (void*)&sub_flow, (void*)&sub_status, (void*)&n_pts, (void*)&iters,
                         (void*)&c0, (void*)&c_min, (void*)&affine, (void*)&partial, (void*)&dev_status};
         const unsigned grid = dgf::cooperative_blocks(gm_fit_kernel, kPartThreads, kParts);
-        if (grid < 1) return DGF_ERR_CUDA;
-        if (cudaLaunchCooperativeKernel((const void*)gm_fit_kernel, dim3(grid), dim3(kPartThreads), args, 0, stream) !=
-            cudaSuccess)
-            return DGF_ERR_CUDA;
+        if ((rc = dgf::launch_cooperative((const void*)gm_fit_kernel, grid, dim3(kPartThreads), args, stream)) != DGF_OK)
+            return rc;
     }
-    if ((rc = dgf::launch_status()) != DGF_OK) return rc;
     // 3. main pass from the prior
     main.pyr_levels = pyr_levels;
     main.n_jobs = 1;

@@ -25,12 +25,24 @@ extern "C" int fit(int blocks, const float* pts, int stride, const float* flow, 
         return DGF_ERR_CUDA;
     return cudaDeviceSynchronize() == cudaSuccess ? DGF_OK : DGF_ERR_CUDA;
 }
+// A launch on more blocks than fit the device, which the runtime refuses: the status, and that of a check afterwards.
+extern "C" void refused(int* out)
+{
+    int n = 0, stride = 1, iters = 1;
+    double c0 = 1.0, c_min = 1.0;
+    void* null = nullptr;
+    void* args[] = {&null, &stride, &null, &null, &n, &iters, &c0, &c_min, &null, &null, &null};
+    out[0] = dgf::launch_cooperative((const void*)gm_fit_kernel, 1u << 20, dim3(kPartThreads), args, 0);
+    out[1] = dgf::launch_status();
+    out[2] = dgf::launch_cooperative((const void*)gm_fit_kernel, 0, dim3(kPartThreads), args, 0);
+    out[3] = dgf::launch_status();
+}
 extern "C" size_t partial_bytes() { return kPartialBytes; }
 """
 
 
 @pytest.fixture(scope="module")
-def fit(tmp_path_factory):
+def lib(tmp_path_factory):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     import paper_1901_09971_gb300 as dgf
@@ -43,7 +55,11 @@ def fit(tmp_path_factory):
                     "-Xlinker", os.path.dirname(build.LIB), "-o", out], check=True, capture_output=True)
     lib = ctypes.CDLL(out)
     lib.partial_bytes.restype = ctypes.c_size_t
+    return lib
 
+
+@pytest.fixture(scope="module")
+def fit(lib):
     def run(blocks, pts, stride, flow, status, n, iters):
         state = torch.zeros(32, dtype=torch.float64, device="cuda")
         partial = torch.full((lib.partial_bytes() // 8,), float("nan"), dtype=torch.float64, device="cuda")
@@ -74,3 +90,9 @@ def test_any_number_of_blocks_gives_the_same_fit(fit, n):
     assert np.isfinite(ref[:6]).all() and ref[6:].view(np.int32)[0] == 1
     for blocks in (63, 32, 17, 8, 3, 2, 1):
         np.testing.assert_array_equal(fit(blocks, pts, stride, flow, status, n, iters).view(np.uint64), ref.view(np.uint64))
+
+
+def test_a_refused_launch_does_not_fail_the_next_call(lib):
+    out = (ctypes.c_int * 4)()
+    lib.refused(out)
+    assert out[0] != 0 and out[1] == 0 and out[2] != 0 and out[3] == 0
