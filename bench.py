@@ -174,7 +174,7 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(self.rows)}
 
 
-TRAFFIC_SOURCES = ("rlof.cu", "common.cuh", "batch.cuh")  # what the tracking kernel is compiled from
+TRAFFIC_SOURCES = ("rlof.cu", "track_index.cuh", "common.cuh", "batch.cuh")  # what the tracking kernel is compiled from
 
 
 def tracking_sources_digest():
@@ -783,7 +783,9 @@ def run_cuda(args, rank: int, world: int, local_rank: int):
                              "peak_basis": f"measured: FP32 FMA probe (dgf_fp32_probe, the faster of scalar and "
                                            f"packed FMA) on {fp32['sms']} SMs at a median {fp32['sm_mhz']} MHz, "
                                            f"CUDA events",
-                             "kernel": "rlof_kernel", "flops_per_launch": flops},
+                             "kernel": "rlof_kernel", "flops_per_launch": flops,
+                             "flops_basis": "every iteration counted as a full step; a step whose residuals all "
+                                            "have weight 1 (18% of this pair's) does about two thirds of it"},
                 "fp32_peak": fp32,
                 "e2e": {"value": e2e_value, "unit": "points/s", "h2d_bytes_per_step": 2 * W * H,
                         "d2h_bytes_per_step": n_pts * (8 + 8 + 1)},

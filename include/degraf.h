@@ -72,7 +72,9 @@ int dgf_version(void);
  * stream: detection and the pyramid stage frame rows with bulk asynchronous copies
  * when the frame's base, pitch and width are multiples of 16, and a block whose
  * copies never complete gives up after a bounded wait and leaves its outputs
- * unwritten; epic_interpolate reports a labelling that did not settle and a search
+ * unwritten; a block of rlof_track_gm's fit that waits in vain for the others reports
+ * it in the same way (its main pass then starts from what was fitted so far);
+ * epic_interpolate reports a labelling that did not settle and a search
  * that outgrew its layout (its dense field is then incomplete). reset = 1 also
  * clears the word. Synchronous: waits for the device's pending work. The first
  * call on a device, or the first launch of those kernels, looks the word's address

@@ -136,9 +136,11 @@ class EpicParams:
 
 
 def device_status(reset: bool = False) -> int:
-    """Thread blocks of detection or the pyramid that gave up waiting for their
-    staging copies on the current device since the last reset (0: every launch ran
-    to the end). Synchronises the device."""
+    """DGF_DEV_* bits of the device-side failures on the current device since the last
+    reset (0: every launch ran to the end): 1, a block of detection or the pyramid gave
+    up waiting for its staging copies, or one of the global-motion fit for the others; 2,
+    EPIC's labelling did not settle; 4, a neighbourhood search of EPIC outgrew its
+    largest layout. Synchronises the device."""
     v = ctypes.c_uint(0)
     check("dgf_device_status", load().dgf_device_status(ctypes.byref(v), int(reset)))
     return int(v.value)

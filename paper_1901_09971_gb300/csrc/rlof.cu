@@ -56,7 +56,8 @@ __host__ __device__ constexpr int block_threads()
 // registers all the same (16 blocks fit) give faster code: 13 one-warp blocks at radius
 // 5 (the 1242x375 pair's whole pass 1.119, 1.082, 1.089 and 1.098 ms with bounds of 12,
 // 13, 14 and 16), 14 at radius 4 with the square support (16 mixed pairs 4.956 against
-// 4.977 ms with 16; with the cross support 583 against 577 us, so 16 there).
+// 4.977 ms with 16; with the cross support 583 against 577 us, so 16 there). In FP32 with
+// the square support both still spill some 60 to 120 bytes a thread.
 template <int G, int RC, bool CROSS>
 __host__ __device__ constexpr int min_blocks()
 {
@@ -737,9 +738,11 @@ __device__ __forceinline__ void accumulate(const Support<SLP>& S, const TT& tt, 
         static_assert(RL::slots == SLP, "run layout slot count");
         // the generic slots' samples first, where their unswapped bilinear weights would
         // otherwise hold registers during the runs (radius 4, 16 mixed pairs 5.03 -> 4.95
-        // ms); the other instantiations measured faster with them last (radius 5 on a
-        // 1257x566 pair 1.572 against 1.600 ms). Their terms are added last, in slot
-        // order; a slot past the support reads the block's first taps.
+        // ms); last at radius 5 (a 1257x566 pair 1.572 against 1.600 ms with them first)
+        // and with the cross support (1242x375 580 against 585 us). Translation-only
+        // tracking at radius 4 would gain from first too (1257x566 358 -> 349 us) and has
+        // them last so far. Their terms are added last, in slot order; a slot past the
+        // support reads the block's first taps.
         constexpr bool kEarly = RC == 4 && MODEL == 4 && !CROSS;
         auto generic_slot = [&](int j) {
             // the radius-4 run layout's generic slot holds vertical pairs only
@@ -891,8 +894,11 @@ __device__ __forceinline__ void cross_arms(const LevelView<TS>& L, float plx, fl
 // matrix. One plane after the other and each without a branch, so that the loads of a
 // plane (and of the next, as registers allow) are in flight together, a run's tap rows
 // read once: a level's set-up waits for a few memory latencies instead of one for
-// every slot (3,500 instead of 5,600 cycles on the 64-pair batch's frames). With the cross
-// support's masks the other form measured faster (591 against 600 us at radius 4).
+// every slot (3,500 instead of 5,600 cycles on the 64-pair batch's frames; 16 mixed pairs
+// 5.00 -> 4.96 ms). Used where it was first measured, model 4 in FP32 without the cross
+// support's masks, with which the other form is faster (591 against 600 us at radius 4).
+// Half storage has the other form so far, although it would gain at radius 4 (1257x566
+// 453 -> 441 us) and is level at radius 5; translation-only tracking is level.
 template <typename TS, int G, int SLP, int RC>
 __device__ __forceinline__ void run_template(Support<SLP>& S, const LevelView<TS>& L, int bx, int by,
                                              const PairWeights& pw, bool direct, int lane, float2& g00, float2& g01,
@@ -1190,8 +1196,11 @@ struct FactorOf<2> {
 // Short steps (model 4): while every residual of a point stays at or below r_in, where
 // the Hampel weight is exactly 1, the normal matrix depends on the template alone. A
 // full step whose weights sum up to the support's samples predicts that of the next
-// step, and the last step of the level above of a level's first (with the cross
-// support, whose supports differ from level to level, only a later step does); once
+// step, and the last step of a level that of the level below's first, also with the
+// cross support, though its supports differ from level to level (there a full first
+// step of a level predicts nothing, later ones do: translations on 1257x566 at radius 5
+// take 723 us a pass, against 746 when every full step predicts within its level and
+// none across levels; 1242x375 at radius 4 580 and 581). Once
 // every group of the warp that still iterates predicts it, the groups form the four
 // sums of the right-hand side only, about two thirds of a full step's instructions
 // (no weights, 4 of 14 sums, no factorisation), and solve with the factored
@@ -1203,11 +1212,17 @@ struct FactorOf<2> {
 // vote after every step cost 8-11% where no step was short, and without a vote among
 // short steps a group that had failed waited for the longest of the others (14% on a
 // pair of large motion). What a point needs once a level (its position, its start
-// displacement) waits in shared memory, for the registers. Measured, whole passes: 16
-// mixed pairs (radius 4, translations, 94% of the steps short) 6.42 -> 4.96 ms; the
-// 1242x375 pair (radius 5, large motion, 18%) 1.083 -> 1.075; 1257x566 with large motion
-// 1.577 -> 1.577 at radius 5 and 1.288 -> 1.309 at radius 4. Translation-only tracking
-// has 5 sums; leaving out 3 gained nothing.
+// displacement) waits in shared memory, for the registers. Measured with the set-up
+// below and the register bounds above, whole passes: 16 mixed pairs (radius 4,
+// translations, 94% of the steps short) 6.42 -> 4.96 ms; the 1242x375 pair (radius 5,
+// large motion, 18%) 1.083 -> 1.071. What few steps are short on costs: large motion on
+// 1257x566 1.578 -> 1.571 at radius 5, 1.289 -> 1.311 at radius 4; on 651x366, whose
+// points are all resident at once, 160 -> 164 us at radius 5, 136 -> 142 at radius 4.
+// At radius 4 most of it is register spills and order of loads, not votes (without
+// votes 140 us); leaving the votes for a warp's remaining levels once a level had no
+// short step, or a failed one, gave no more than it lost elsewhere (651x366 141.6 us,
+// 256x128 pair 71 -> 75). Translation-only tracking has 5 sums; leaving out 3 gained
+// nothing.
 template <typename TS, int G, int SLP, int MODEL, int MINB, int RC, bool CROSS>
 __global__ void __launch_bounds__(block_threads<G>(), MINB) rlof_kernel(const __grid_constant__ TrackBatch a)
 {
